@@ -49,35 +49,35 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr float kSubScale = 1099511627776.f;        // 2^40
 constexpr float kSubUnit = 9.094947017729282e-13f;  // 2^-40
 
-// Lanes that work on one ray: G = 16 (half a warp) or 32.
+// Lanes that work on one ray: G = 16 (half a warp) or 32. Every member is called by the whole
+// warp together: with G = 16 the warp's two rays run in lock-step, each instruction issued once
+// for both (votes and shuffles take the full mask and stay inside the group by their width).
 template <int G>
 struct Grp {
-  unsigned mask;  // the group's lanes in the warp
   int lane;       // lane within the group
   int base;       // warp lane of the group's lane 0
-  __device__ unsigned ballot(bool p) const { return __ballot_sync(mask, p) >> base; }
-  __device__ unsigned below() const { return (1u << lane) - 1u; }
-  __device__ float sum(float v) const {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_down_sync(mask, v, o, G);
-    return __shfl_sync(mask, v, 0, G);  // group lane 0's sum, identical on every lane
+  __device__ unsigned ballot(bool p) const {
+    const unsigned b = __ballot_sync(kFull, p) >> base;
+    return G == 32 ? b : b & ((1u << (G & 31)) - 1u);
   }
-  __device__ long long sum(long long v) const {
+  __device__ unsigned below() const { return (1u << lane) - 1u; }
+  __device__ long long sum(long long v) const {  // integer: the same in any order
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_down_sync(mask, v, o, G);
-    return __shfl_sync(mask, v, 0, G);
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o, G);
+    return v;
   }
   __device__ float max(float v) const {
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(mask, v, o, G));
+    for (int o = G / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kFull, v, o, G));
     return v;
   }
   template <class T>
-  __device__ T shfl(T v, int src) const { return __shfl_sync(mask, v, src, G); }
-  template <class T>
-  __device__ T shfl_xor(T v, int o) const { return __shfl_xor_sync(mask, v, o, G); }
-  __device__ void sync() const { __syncwarp(mask); }
-  __device__ unsigned total(unsigned v) const { return __reduce_add_sync(mask, v); }
+  __device__ T shfl_xor(T v, int o) const { return __shfl_xor_sync(kFull, v, o, G); }
+  __device__ unsigned total(unsigned v) const {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o, G);
+    return v;
+  }
 };
 
 // Interval columns of one ray (cap entries each). For the interval clipped to the bracket,
@@ -127,10 +127,11 @@ struct Finish {
 
 // Root of F = u on [lo, min(hi, last interval end)] over the n collected intervals, then the
 // race at t_u. The sums are fixed-point integers, so the result does not depend on G or on the
-// order of the intervals.
+// order of the intervals. Called by the whole warp; a group without a ray passes act = false and
+// n = 0 and follows along.
 template <int G>
 __device__ Finish solve(const Grp<G>& g, const Iv& iv, int n, float lo, float hi, float Flo, float u, float u2,
-                        float t1, int spawn_mode) {
+                        float t1, int spawn_mode, bool act) {
   const int lane = g.lane;
   Finish out{-1, t1, t1, UGP_RAY_OK};
   float bmax = lo, emax = 0.f;
@@ -156,9 +157,9 @@ __device__ Finish solve(const Grp<G>& g, const Iv& iv, int n, float lo, float hi
     const float tq = tau_at(t, iv.tn[e], iv.ts[e], iv.s[e]);
     return iv.e0[e] * (0.25f * kSqrtPi) / iv.s[e] * cut_diff(iv.ex0[e], erfcf(fabsf(tq)), tq);
   };
-  auto evalF = [&](float t, float& f, float& fp) {
+  auto evalF = [&](float t, int m, float& f, float& fp) {
     long long fl = 0, fpl = 0;
-    for (int e = lane; e < n; e += G) {
+    for (int e = lane; e < m; e += G) {
       const float a = iv.a[e], b = iv.b[e];
       fl += fxF(b <= t ? full[e] : term(e, t));
       if (a <= t && t <= b) fpl += __float2ll_rn(0.5f * gauss_at(t, iv.tn[e], iv.ts[e], iv.s[e], iv.e0[e]) * dscale);
@@ -172,66 +173,75 @@ __device__ Finish solve(const Grp<G>& g, const Iv& iv, int n, float lo, float hi
     for (int e = lane; e < n; e += G) fl += fxF(full[e]);
     fh = Flo - u + float(g.sum(fl)) * kFUnit;
   }
-  float t;
-  if (!(fh > 0.f)) {
-    t = hi_e;  // rounding placed the crossing at the end of the bracket
-  } else {
-    // Newton's method safeguarded by a bracket [a0, b0] with f(a0) < 0 < f(b0); a step that
-    // leaves the bracket or does not shrink fast enough is replaced by a false-position step
-    // with the Illinois rule (F is monotone and S-shaped across thin primitives, where plain
-    // Newton overshoots and bisection would crawl)
-    float a0 = lo, b0 = hi_e, fa = Flo - u, fb = fh;
-    int moved = 0;  // -1: a0 moved last, +1: b0 moved last
+  float t = hi_e;  // kept when rounding placed the crossing at the end of the bracket
+  // Newton's method safeguarded by a bracket [a0, b0] with f(a0) < 0 < f(b0); a step that
+  // leaves the bracket or does not shrink fast enough is replaced by a false-position step
+  // with the Illinois rule (F is monotone and S-shaped across thin primitives, where plain
+  // Newton overshoots and bisection would crawl)
+  bool run = act && fh > 0.f;
+  float a0 = lo, b0 = hi_e, fa = Flo - u, fb = fh;
+  int moved = 0;  // -1: a0 moved last, +1: b0 moved last
+  if (run) {
     t = a0 - fa * (b0 - a0) / (fb - fa);
     if (!(t > a0 && t < b0)) t = 0.5f * (a0 + b0);
-    float dx_old = b0 - a0, dx = dx_old;
-    bool conv = false;
-    for (int it = 0; it < kDNewton; ++it) {
-      float f, fp;
-      evalF(t, f, fp);
-      if (f == 0.f) { conv = true; break; }
-      if (f < 0.f) {
-        a0 = t;
-        fa = f;
-        if (moved < 0) fb *= 0.5f;
-        moved = -1;
-      } else {
-        b0 = t;
-        fb = f;
-        if (moved > 0) fa *= 0.5f;
-        moved = 1;
-      }
-      if (!(nextafterf(a0, INFINITY) < b0)) { conv = true; break; }
-      // a Newton correction below 1e-6 of the distance scale ends the iteration: its own error
-      // is of the order of its square (or of itself across a kink of F'), far below the 1e-5
-      // accuracy asked (taken even where the shrink safeguard below would refuse the step,
-      // which near the root only reflects the rounding noise of f)
-      if (fp > 0.f && fabsf(f) <= kNewtonStep * fmaxf(fabsf(t), kNewtonFloor) * fp) {
-        const float tn = t - f / fp;
-        if (tn > a0 && tn < b0) t = tn;
-        conv = true;
-        break;
-      }
-      const float tn = fp > 0.f ? t - f / fp : a0;
-      float tnew;
-      // past kDBisectAfter steps only bisection: the bracket then collapses to adjacent floats
-      // within the iteration bound, whatever F looks like
-      const bool bisect = it >= kDBisectAfter;
-      if (!bisect && fp > 0.f && tn > a0 && tn < b0 && fabsf(2.f * f) <= fabsf(dx_old * fp)) {
-        dx_old = dx;
-        dx = f / fp;
-        tnew = tn;
-      } else {
-        tnew = bisect ? 0.5f * (a0 + b0) : a0 - fa * (b0 - a0) / (fb - fa);
-        if (!(tnew > a0 && tnew < b0)) tnew = 0.5f * (a0 + b0);
-        dx_old = dx;
-        dx = tnew - t;
-      }
-      if (tnew == t) { conv = true; break; }
-      t = tnew;
-    }
-    if (!conv) out.st = UGP_RAY_SOLVE_LIMIT;
   }
+  float dx_old = b0 - a0, dx = dx_old;
+  for (int it = 0; it < kDNewton; ++it) {
+    if (!__any_sync(kFull, run)) break;
+    float f, fp;
+    evalF(t, run ? n : 0, f, fp);
+    if (!run) continue;
+    if (f == 0.f) {
+      run = false;
+      continue;
+    }
+    if (f < 0.f) {
+      a0 = t;
+      fa = f;
+      if (moved < 0) fb *= 0.5f;
+      moved = -1;
+    } else {
+      b0 = t;
+      fb = f;
+      if (moved > 0) fa *= 0.5f;
+      moved = 1;
+    }
+    if (!(nextafterf(a0, INFINITY) < b0)) {
+      run = false;
+      continue;
+    }
+    // a Newton correction below 1e-6 of the distance scale ends the iteration: its own error
+    // is of the order of its square (or of itself across a kink of F'), far below the 1e-5
+    // accuracy asked (taken even where the shrink safeguard below would refuse the step,
+    // which near the root only reflects the rounding noise of f)
+    if (fp > 0.f && fabsf(f) <= kNewtonStep * fmaxf(fabsf(t), kNewtonFloor) * fp) {
+      const float tn = t - f / fp;
+      if (tn > a0 && tn < b0) t = tn;
+      run = false;
+      continue;
+    }
+    const float tn = fp > 0.f ? t - f / fp : a0;
+    float tnew;
+    // past kDBisectAfter steps only bisection: the bracket then collapses to adjacent floats
+    // within the iteration bound, whatever F looks like
+    const bool bisect = it >= kDBisectAfter;
+    if (!bisect && fp > 0.f && tn > a0 && tn < b0 && fabsf(2.f * f) <= fabsf(dx_old * fp)) {
+      dx_old = dx;
+      dx = f / fp;
+      tnew = tn;
+    } else {
+      tnew = bisect ? 0.5f * (a0 + b0) : a0 - fa * (b0 - a0) / (fb - fa);
+      if (!(tnew > a0 && tnew < b0)) tnew = 0.5f * (a0 + b0);
+      dx_old = dx;
+      dx = tnew - t;
+    }
+    if (tnew == t) {
+      run = false;
+      continue;
+    }
+    t = tnew;
+  }
+  if (run) out.st = UGP_RAY_SOLVE_LIMIT;
   // race: smallest E_k / G_k(x_t) among the intervals containing t (ties: smaller index)
   float best = INFINITY;
   int best_id = INT32_MAX, best_e = -1;
@@ -264,17 +274,15 @@ __device__ Finish solve(const Grp<G>& g, const Iv& iv, int n, float lo, float hi
 }
 
 // Tests candidate `slot` (< 0: none) on every lane of the group and appends the hits meeting
-// [lo, hi] to iv (at most iv.cap are stored); n counts all of them.
+// [lo, hi] to iv (at most iv.cap are stored); n counts all of them. Called by the whole warp.
 template <int G>
 __device__ __forceinline__ void collect_one(const Grp<G>& g, const Iv& iv, const TraceScene& sc, const Ray& ray,
                                             float lo, float hi, float t0, float t1, int excl, int slot, int& n,
                                             unsigned& np) {
   PrimHit hh;
-  bool ok = false;
-  if (slot >= 0) {
-    ++np;
-    ok = prim_test(sc.prims, sc.wlo, slot, ray, t0, t1, sc.k2, excl, hh) && fmaxf(hh.a, lo) < fminf(hh.b, hi);
-  }
+  np += slot >= 0 ? 1u : 0u;
+  const bool ok = prim_test_of<true>(slot >= 0, sc.prims, sc.wlo, slot, ray, t0, t1, sc.k2, excl, hh) &&
+                  fmaxf(hh.a, lo) < fminf(hh.b, hi);
   const unsigned m = g.ballot(ok);
   if (ok) {
     const int i = n + __popc(m & g.below());
@@ -404,7 +412,7 @@ __global__ void __launch_bounds__(32 * kDWarps) k_dense(TraceScene sc0, DenseQue
   extern __shared__ __align__(16) unsigned char dsm[];
   WarpSmem& W = reinterpret_cast<WarpSmem*>(dsm)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31, half = lane >> 4;
-  const Grp<kHalf> g{0xffffu << (16 * half), lane & 15, 16 * half};
+  const Grp<kHalf> g{lane & 15, 16 * half};
   const Iv iv = W.iv.view(half * kDCap, kDCap);
   const int count = n_dev ? *reinterpret_cast<const volatile int*>(n_dev) : int(n_host);
   const int nwarps = gridDim.x * kDWarps;
@@ -412,19 +420,21 @@ __global__ void __launch_bounds__(32 * kDWarps) k_dense(TraceScene sc0, DenseQue
   // table are in flight together
   for (int p = blockIdx.x * kDWarps + (threadIdx.x >> 5); 2 * p < count; p += nwarps) {
     const int j = 2 * p + half;
-    if (j >= count || __ldg(q.idx + j) < 0) continue;
-    const RayIn R = ray_in(sc0, q, j);
-    bool big = R.list == nullptr;
+    bool act = j < count && __ldg(q.idx + j) >= 0;
+    if (!__any_sync(kFull, act)) continue;
+    RayIn R{};
+    if (act) R = ray_in(sc0, q, j);
+    bool big = act && R.list == nullptr;
+    const int nl = act && !big ? R.nlist : 0;
+    const int nl_max = max(nl, __shfl_xor_sync(kFull, nl, kHalf));
     int n = 0;
     unsigned np = 0;
-    if (!big) {
-      for (int base = 0; base < R.nlist; base += kHalf) {
-        const int e = base + g.lane;
-        collect_one(g, iv, R.sc, R.ray, R.lo, R.hi, R.t0, R.t1, R.excl, e < R.nlist ? __ldg(R.list + e) : -1, n, np);
-      }
-      g.sync();
-      big = n > kDCap;
+    for (int base = 0; base < nl_max; base += kHalf) {
+      const int e = base + g.lane;
+      collect_one(g, iv, R.sc, R.ray, R.lo, R.hi, R.t0, R.t1, R.excl, e < nl ? __ldg(R.list + e) : -1, n, np);
     }
+    __syncwarp();
+    big = big || n > kDCap;
     const unsigned tp = g.total(np);
     if (big) {  // k_dense_big rebuilds and finishes the ray
       if (g.lane == 0) {
@@ -434,12 +444,13 @@ __global__ void __launch_bounds__(32 * kDWarps) k_dense(TraceScene sc0, DenseQue
           atomicAdd(O.stats + 5, 1ull);
         }
       }
-      g.sync();
-      continue;
+      act = false;
+      n = 0;
     }
-    const Finish f = solve(g, iv, n, R.lo, R.hi, R.Flo, R.u, R.u2, R.t1, O.spawn_mode);
-    if (g.lane == 0) write_out(O, R.idx, f, 0u, tp);
-    g.sync();
+    __syncwarp();
+    const Finish f = solve(g, iv, n, R.lo, R.hi, R.Flo, R.u, R.u2, R.t1, O.spawn_mode, act);
+    if (act && g.lane == 0) write_out(O, R.idx, f, 0u, tp);
+    __syncwarp();
   }
 }
 
@@ -453,7 +464,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_dense_big(TraceScene sc0, Dense
   extern __shared__ __align__(16) unsigned char dsm[];
   WarpSmemBig& W = reinterpret_cast<WarpSmemBig*>(dsm)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  const Grp<32> gw{kFull, lane, 0};
+  const Grp<32> gw{lane, 0};
   // this warp's interval slot (the grid has at most q.big_slots warps)
   float* slot = q.big_iv + size_t(blockIdx.x * kWarps + (threadIdx.x >> 5)) * (size_t(kCap) * 9);
   const Iv iv{slot, slot + kCap, slot + 2 * kCap, slot + 3 * kCap, slot + 4 * kCap, slot + 5 * kCap,
@@ -484,7 +495,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_dense_big(TraceScene sc0, Dense
       if (st != UGP_RAY_OK) break;
       if (n <= kCap) {
         // ---- 2. the solve
-        f = solve(gw, iv, n, lo, hi, Flo, R.u, R.u2, R.t1, O.spawn_mode);
+        f = solve(gw, iv, n, lo, hi, Flo, R.u, R.u2, R.t1, O.spawn_mode, true);
         done = true;
       } else if (next_count && level == 0) {
         handed = true;  // the next pass holds more intervals

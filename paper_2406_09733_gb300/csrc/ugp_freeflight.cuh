@@ -178,14 +178,12 @@ struct OwnerRay {
   __device__ float edge(int j) const { return bin_edge(lo, hi, L, j); }
 };
 
-// Tests primitive `slot` against the owner's ray and adds its interval's contribution to the
+// Adds the interval `h` of primitive `slot` on the owner's ray to the
 // owner's bins up to the owner's crossing bin, with shared-memory atomics (other lanes may bin
 // primitives of the same ray in the same step); contributions to bins before the crossing bin
 // also go to the owner's running sum of them, and a primitive met before the crossing bin's end
 // goes into the owner's slot list. The owner moves its crossing bin afterwards.
-static __device__ void pooled_leaf(FFSmem& sm, const OwnerRay& w, int slot) {
-  PrimHit h;
-  if (!prim_test(w.prims, w.wlo, slot, w.ray, w.t0, w.t1, w.k2, w.ex, h)) return;
+static __device__ void pooled_leaf(FFSmem& sm, const OwnerRay& w, int slot, const PrimHit& h) {
   const float x = fmaxf(h.a, w.lo), y = fminf(h.b, w.hi);
   if (!(x < y)) return;
   int j = min(kB - 1, max(0, int(float(kB) * sqrtf((x - w.lo) / w.L))));
@@ -349,7 +347,9 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
       w.jc = __shfl_sync(kFull, jc, o);
       w.list = reinterpret_cast<int*>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(c.list), o));
       w.tid = (int(threadIdx.x) & ~31) | o;
-      if (work) pooled_leaf(sm, w, sm.lq[nq_o - 1 - (lane - off_o)][w.tid]);
+      const int slot = work ? sm.lq[nq_o - 1 - (lane - off_o)][w.tid] : 0;
+      PrimHit h;
+      if (prim_test_of<true>(work, w.prims, w.wlo, slot, w.ray, w.t0, w.t1, w.k2, w.ex, h)) pooled_leaf(sm, w, slot, h);
       __syncwarp();
       // each ray drops the items taken from the top of its queue and, when its running sum of
       // the bins before the crossing bin passes u, moves the crossing bin (bins are
