@@ -335,13 +335,23 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_b_shadow(BState S)
   const BPaths& P = S.P;
   // one ray per thread over a grid sized for the pool: the hardware spreads the blocks
   const int j = int(blockIdx.x * blockDim.x + threadIdx.x);
-  if (j >= count) return;
-  const int p = S.sh.path[j];
-  const TraceScene sc = S.scenes[P.req[p]];
-  const Ray ray = make_ray(f3(S.sh.ox[j], S.sh.oy[j], S.sh.oz[j]), f3(S.sh.dx[j], S.sh.dy[j], S.sh.dz[j]));
+  if ((j & ~31) >= count) return;  // the whole warp
+  const bool live = j < count;
   TrStats ts{0u, 0u, UGP_RAY_OK};
-  const float tau = tr_optical_depth(sc, ray, 0.f, S.sh.dist[j], S.sh.excl[j], stk + threadIdx.x, kTrBlock,
-                                     tr_acc + threadIdx.x, tr_owner + threadIdx.x, ts);
+  TraceScene sc{};
+  Ray ray{};
+  float dist = 0.f;
+  int p = 0, ex = -1;
+  if (live) {
+    p = S.sh.path[j];
+    sc = S.scenes[P.req[p]];
+    ray = make_ray(f3(S.sh.ox[j], S.sh.oy[j], S.sh.oz[j]), f3(S.sh.dx[j], S.sh.dy[j], S.sh.dz[j]));
+    dist = S.sh.dist[j];
+    ex = S.sh.excl[j];
+  }
+  const float tau = tr_optical_depth(sc, ray, 0.f, dist, ex, stk + threadIdx.x, kTrBlock, tr_acc + threadIdx.x,
+                                     tr_owner + threadIdx.x, ts, live);
+  if (!live) return;
   const float T = fmaxf(0.f, 1.f - tau);
   if (T > 0.f) {
     P.ps.lr[p] += T * S.sh.cr[j];

@@ -297,12 +297,15 @@ __device__ __forceinline__ float tau_at(float t, float tn, float ts, float s) { 
 // with sqrt(pi / 2A) = sqrt(pi) / (2 s).  Same-sign arguments use erfc to avoid cancellation.
 __device__ __forceinline__ float half_integral_tau(float tx, float ty, float s, float e0) {
   float diff;
-  if (tx >= 0.f)
-    diff = erfcf(tx) - erfcf(ty);
-  else if (ty <= 0.f)
-    diff = erfcf(-ty) - erfcf(-tx);
-  else
-    diff = erff(ty) - erff(tx);
+  if (tx >= 0.f || ty <= 0.f) {
+    const float u = tx >= 0.f ? tx : -ty, v = tx >= 0.f ? ty : -tx;
+    diff = erfcf(u) - erfcf(v);
+  } else {
+    // most intervals run from the ellipsoid's entry to its exit, tx = -ty: one erf (an odd
+    // function) serves both ends
+    const float e = erff(ty);
+    diff = e - (tx == -ty ? -e : erff(tx));
+  }
   return e0 * (0.25f * kSqrtPi) / s * diff;
 }
 

@@ -338,14 +338,22 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_shadow(TraceScene 
   if (blockIdx.x == 0 && threadIdx.x == 0 && rays) atomicAdd(rays + 1, (unsigned long long)count);
   // one ray per thread over a grid sized for the longest queue: the hardware spreads the blocks
   const int j = int(blockIdx.x * blockDim.x + threadIdx.x);
-  if (j >= count) return;
-  const Ray ray = make_ray(f3(sh.ox[j], sh.oy[j], sh.oz[j]), f3(sh.dx[j], sh.dy[j], sh.dz[j]));
+  if ((j & ~31) >= count) return;  // the whole warp
+  const bool live = j < count;
   TrStats ts{0u, 0u, UGP_RAY_OK};
+  Ray ray{};
+  float dist = 0.f;
+  int ex = -1;
+  if (live) {
+    ray = make_ray(f3(sh.ox[j], sh.oy[j], sh.oz[j]), f3(sh.dx[j], sh.dy[j], sh.dz[j]));
+    dist = sh.dist[j];
+    ex = sh.excl[j];
+  }
   // a negative distance marks a light sample of an emissive primitive: it counts when the
   // point lies before saturation (T > 0) and is not scaled by T
-  const float dist = sh.dist[j];
-  const float tau = tr_optical_depth(sc, ray, 0.f, fabsf(dist), sh.excl[j], stk + threadIdx.x, kTrBlock,
-                                     tr_acc + threadIdx.x, tr_owner + threadIdx.x, ts);
+  const float tau = tr_optical_depth(sc, ray, 0.f, fabsf(dist), ex, stk + threadIdx.x, kTrBlock,
+                                     tr_acc + threadIdx.x, tr_owner + threadIdx.x, ts, live);
+  if (!live) return;
   const float T = fmaxf(0.f, 1.f - tau);
   if (T > 0.f) {
     const float s = dist < 0.f ? 1.f : T;

@@ -21,11 +21,20 @@ k_transmittance(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, con
   __shared__ unsigned long long tr_acc[kTrBlock];
   __shared__ int tr_owner[kTrBlock];
   const int64_t r = int64_t(blockIdx.x) * kTrBlock + threadIdx.x;
-  if (r >= n_rays) return;
+  const bool live = r < n_rays;
   TrStats ts{0u, 0u, UGP_RAY_OK};
-  const float acc = tr_optical_depth(sc, make_ray(ld3(o3, r), ld3(d3, r)), __ldg(t0a + r), __ldg(t1a + r),
-                                     excl ? __ldg(excl + r) : -1, stk + threadIdx.x, kTrBlock, tr_acc + threadIdx.x,
-                                     tr_owner + threadIdx.x, ts);
+  Ray ray{};
+  float t0 = 0.f, t1 = 0.f;
+  int ex = -1;
+  if (live) {
+    ray = make_ray(ld3(o3, r), ld3(d3, r));
+    t0 = __ldg(t0a + r);
+    t1 = __ldg(t1a + r);
+    if (excl) ex = __ldg(excl + r);
+  }
+  const float acc = tr_optical_depth(sc, ray, t0, t1, ex, stk + threadIdx.x, kTrBlock, tr_acc + threadIdx.x,
+                                     tr_owner + threadIdx.x, ts, live);
+  if (!live) return;
   T_out[r] = fmaxf(0.f, 1.f - acc);
   if (st_out) st_out[r] = ts.st;
   if (STATS) add_counters(ctr, ts.n_nodes, ts.n_prims, 1u, 1u, 0u);
