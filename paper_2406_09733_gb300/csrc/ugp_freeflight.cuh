@@ -32,7 +32,7 @@
 //    argmin across them.
 //
 // The scan runs on persistent lanes: a lane whose ray is done takes a new one, and the idle
-// lanes of a warp fetch together (one atomic) once kRefill of them are idle, so a warp does not
+// lanes of a warp write out and fetch together (one atomic) once kRefill of them are idle, so a warp does not
 // wait for its slowest ray before starting new ones (per-ray work varies several-fold; on camera
 // rays of a 1M-primitive room the mean over a warp is 0.58 of its maximum). Each loop step is
 // either a node step (every lane with nodes left visits one) or a leaf step: primitives met in
@@ -147,7 +147,11 @@ static __device__ FFResult scan_result(FFSmem& sm, int tid, const ScanState& s, 
 
 #undef FB
 
-constexpr int kRefill = 2;  // idle lanes of a warp that trigger a joint fetch of new rays
+// Lanes of a warp without a ray (or with a finished one) that trigger a joint write-out and fetch of
+// new rays. Both are code that only those lanes run, about 400 instructions, so several share it:
+// 2^20 camera and bounce rays through a 1M-primitive room 7.58 ms at 2 (fetch only, each ray
+// written as it ended), 7.38 at 4, 7.34 at 8, 7.37 at 12.
+constexpr int kRefill = 8;
 
 // Traversal context of one lane: the scene, the ray and its counters, as used by the
 // persistent driver below.
@@ -249,13 +253,35 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
   int node = 0, sp = 0, jc = kB, nq = 0;
   float lo = 0.f, hi = 0.f, L = 0.f, target = 0.f, limit = 0.f;
   for (;;) {
-    const unsigned idle = __ballot_sync(kFull, !busy && !exhausted);
-    unsigned working = __ballot_sync(kFull, busy);
-    if (idle && (__popc(idle) >= kRefill || working == 0)) {
+    // one packed sum: held-back primitives (9 bits), lanes at work, lanes to refill (idle, or done
+    // with a ray that is not written yet), lanes that need a leaf step
+    const bool ready = busy && tdone && nq == 0;
+    const int mine = busy ? nq : 0;
+    // a node step may add four held-back primitives: it runs only while every lane has room
+    const bool need_leaf = busy && (nq > kLeafQ - 4 || (tdone && nq > 0));
+    const unsigned sums = __reduce_add_sync(
+        kFull, unsigned(mine) | (busy && !ready ? 1u << 9 : 0u) | (ready || (!busy && !exhausted) ? 1u << 15 : 0u) |
+                   (need_leaf ? 1u << 21 : 0u));
+    const int total = int(sums & 511u), refill = int((sums >> 15) & 63u);
+    const bool urgent = (sums >> 21) != 0u;
+    bool working = ((sums >> 9) & 63u) != 0u;
+    if (refill >= kRefill || (refill > 0 && !working)) {
+      if (ready) {
+        s.lo = lo;
+        s.hi = hi;
+        s.jc = jc;
+        s.st = c.st;
+        s.n_nodes = c.n_nodes;
+        s.n_prims = c.n_prims;
+        s.nlist = sm.nlist[c.tid];
+        src.finish(s, scan_result(sm, c.tid, s, true));
+        busy = false;
+      }
+      const unsigned idle = __ballot_sync(kFull, !busy && !exhausted);
       int base = 0;
       const int leader = __ffs(idle) - 1;
-      if (lane == leader) base = atomicAdd(next, __popc(idle));
-      base = __shfl_sync(kFull, base, leader);
+      if (lane == leader) base = atomicAdd(next, __popc(idle));  // no lane when all are exhausted
+      base = __shfl_sync(kFull, base, leader & 31);
       if (!busy && !exhausted) {
         const int i = base + __popc(idle & ((1u << lane) - 1u));
         if (i >= n) {
@@ -299,16 +325,12 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
           }
         }
       }
-      working = __ballot_sync(kFull, busy);
+      working = __any_sync(kFull, busy);
     }
-    if (working == 0) {
-      if (__all_sync(kFull, exhausted)) break;
+    if (!working) {
+      if (refill == 0) break;  // every lane exhausted and its last ray written
       continue;
     }
-    const int mine = busy ? nq : 0;
-    const int total = int(__reduce_add_sync(kFull, unsigned(mine)));
-    // a node step may add four held-back primitives: it runs only while every lane has room
-    const bool urgent = __any_sync(kFull, busy && (nq > kLeafQ - 4 || (tdone && nq > 0)));
     if (total > 0 && (total >= 32 || urgent)) {
       // ---- leaf step: the warp's held-back primitives, up to 32, one per lane whichever ray
       // they belong to; lane i takes item i of the lanes' queues laid end to end
@@ -380,7 +402,7 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
       }
       float en[4];
       int ch[4];
-      unsigned hm = node4_test(c.sc.nodes4, node, c.ray, lo, hi, en, ch);
+      unsigned hm = node4_test(c.sc.nodes4, node, c.ray, lo, limit, en, ch);
       ++c.n_nodes;
       float tk[4];
       int rk[4];
@@ -393,7 +415,7 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
         // a primitive's slot is checked here (its record is loaded by slot); a child node's
         // index is checked when it is visited
         if (ch[k] < 0 && unsigned(~ch[k]) >= unsigned(c.sc.n_prims)) c.st = UGP_RAY_BAD_NODE;
-        if (en[k] > limit || c.st != UGP_RAY_OK) continue;
+        if (c.st != UGP_RAY_OK) continue;
         if (ch[k] < 0) {
           ++c.n_prims;
           sm.lq[nq][c.tid] = ~ch[k];  // nq <= kLeafQ - 4 here: a node adds at most four
@@ -429,17 +451,6 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
         --sp;
         node = sm.stk[sp][c.tid];
       }
-    }
-    if (busy && tdone && nq == 0) {
-      s.lo = lo;
-      s.hi = hi;
-      s.jc = jc;
-      s.st = c.st;
-      s.n_nodes = c.n_nodes;
-      s.n_prims = c.n_prims;
-      s.nlist = sm.nlist[c.tid];
-      src.finish(s, scan_result(sm, c.tid, s, true));
-      busy = false;
     }
   }
 }
