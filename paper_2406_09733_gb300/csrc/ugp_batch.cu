@@ -333,10 +333,12 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_b_shadow(BState S)
   __shared__ int tr_owner[kTrBlock];
   const int count = S.ctl->shadow;
   const BPaths& P = S.P;
-  // one ray per thread over a grid sized for the pool: the hardware spreads the blocks
-  const int j = int(blockIdx.x * blockDim.x + threadIdx.x);
-  if ((j & ~31) >= count) return;  // the whole warp
-  const bool live = j < count;
+  // one ray per thread over a grid sized for the pool (fewer per warp when there are few):
+  // the hardware spreads the blocks
+  const int rpw = rays_per_warp(count, min(int(gridDim.x) * (kTrBlock / 32), kTrWarps));
+  const int j0 = int(blockIdx.x * (kTrBlock / 32) + (threadIdx.x >> 5)) * rpw, j = j0 + int(threadIdx.x & 31);
+  if (j0 >= count) return;  // the whole warp
+  const bool live = int(threadIdx.x & 31) < rpw && j < count;
   TrStats ts{0u, 0u, UGP_RAY_OK};
   TraceScene sc{};
   Ray ray{};
@@ -491,9 +493,9 @@ struct WaveGrids {
   int regen, ext, shade, shadow, retire;
 };
 WaveGrids wave_grids(int64_t pool) {
-  const int ext_need = int((pool + kFFBlock - 1) / kFFBlock), ext_cap = scan_grid((const void*)k_b_extend);
+  const int ext_need = int((pool + kFFBlock / 32 - 1) / (kFFBlock / 32)), ext_cap = scan_grid((const void*)k_b_extend);
   return WaveGrids{grid_of((const void*)k_b_regen, 256, pool), ext_need < ext_cap ? ext_need : ext_cap,
-                   grid_of((const void*)k_b_shade, 128, pool), int((pool + kTrBlock - 1) / kTrBlock),
+                   grid_of((const void*)k_b_shade, 128, pool), tr_grid(pool),
                    grid_of((const void*)k_b_retire, 256, pool)};
 }
 

@@ -80,7 +80,7 @@ ugp_status launch_free_flight(const TraceScene& sc, int64_t n, const float* o3, 
   int* next = dq.count + 1;  // the scan's ray counter, in the queue header next to the queue length
   UGP_CUDA_CHECK(cudaMemsetAsync(dq.count, 0, 2 * sizeof(int), stream));
   const void* kern = ctr ? (const void*)k_free_flight<true> : (const void*)k_free_flight<false>;
-  const int64_t need = (n + kFFBlock - 1) / kFFBlock;
+  const int64_t need = (n + kFFBlock / 32 - 1) / (kFFBlock / 32);  // down to one ray per warp (rays_per_warp)
   const int cap = scan_grid(kern);
   const unsigned grid = unsigned(need < cap ? need : cap);
   prof_begin(kStQuery, stream);

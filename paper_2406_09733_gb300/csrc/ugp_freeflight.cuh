@@ -249,7 +249,9 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
   ScanCtx c{sm, int(threadIdx.x), src.scene(), make_ray(make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 1.f)), 0.f,
             0.f, -1, 0u, 0u, UGP_RAY_OK, nullptr};
   ScanState s;
-  bool busy = false, exhausted = false, tdone = false;
+  const int used = rays_per_warp(n, int64_t(gridDim.x) * (kFFBlock / 32));
+  const int refill_at = max(1, min(kRefill, used / 4));
+  bool busy = false, exhausted = lane >= used, tdone = false;
   int node = 0, sp = 0, jc = kB, nq = 0;
   float lo = 0.f, hi = 0.f, L = 0.f, target = 0.f, limit = 0.f;
   for (;;) {
@@ -265,7 +267,7 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
     const int total = int(sums & 511u), refill = int((sums >> 15) & 63u);
     const bool urgent = (sums >> 21) != 0u;
     bool working = ((sums >> 9) & 63u) != 0u;
-    if (refill >= kRefill || (refill > 0 && !working)) {
+    if (refill >= refill_at || (refill > 0 && !working)) {
       if (ready) {
         s.lo = lo;
         s.hi = hi;

@@ -336,10 +336,12 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_shadow(TraceScene 
   __shared__ int tr_owner[kTrBlock];
   const int count = load_count(cnt);
   if (blockIdx.x == 0 && threadIdx.x == 0 && rays) atomicAdd(rays + 1, (unsigned long long)count);
-  // one ray per thread over a grid sized for the longest queue: the hardware spreads the blocks
-  const int j = int(blockIdx.x * blockDim.x + threadIdx.x);
-  if ((j & ~31) >= count) return;  // the whole warp
-  const bool live = j < count;
+  // one ray per thread over a grid sized for the longest queue (fewer per warp when there are
+  // few): the hardware spreads the blocks
+  const int rpw = rays_per_warp(count, min(int(gridDim.x) * (kTrBlock / 32), kTrWarps));
+  const int j0 = int(blockIdx.x * (kTrBlock / 32) + (threadIdx.x >> 5)) * rpw, j = j0 + int(threadIdx.x & 31);
+  if (j0 >= count) return;  // the whole warp
+  const bool live = int(threadIdx.x & 31) < rpw && j < count;
   TrStats ts{0u, 0u, UGP_RAY_OK};
   Ray ray{};
   float dist = 0.f;
@@ -640,9 +642,9 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
       UGP_CUDA_CHECK(cudaMemsetAsync(gs.L.c[9], 0, size_t(RL.E) * 4, st));
   }
   const int g_cam = grid_for((const void*)k_camera, 256, n);
-  const int g_ext = grid_for((const void*)k_extend, kFFBlock, n);
+  const int g_ext = grid_for((const void*)k_extend, kFFBlock, 32 * n);  // down to one ray per warp
   const int g_shade = guide ? grid_for((const void*)k_shade<true>, 128, n) : grid_for((const void*)k_shade<false>, 128, n);
-  const int g_shadow = int((n + kTrBlock - 1) / kTrBlock);
+  const int g_shadow = tr_grid(n);
   const int g_acc = grid_for((const void*)k_accumulate, 256, n);
   for (int si = 0; si < params->spp; ++si) {
     const int sample = params->spp_begin + si;

@@ -20,8 +20,11 @@ k_transmittance(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, con
   __shared__ int stk[kTrStack * kTrBlock];
   __shared__ unsigned long long tr_acc[kTrBlock];
   __shared__ int tr_owner[kTrBlock];
-  const int64_t r = int64_t(blockIdx.x) * kTrBlock + threadIdx.x;
-  const bool live = r < n_rays;
+  const int rpw = rays_per_warp(n_rays, min(int(gridDim.x) * (kTrBlock / 32), kTrWarps));
+  const int64_t r0 = (int64_t(blockIdx.x) * (kTrBlock / 32) + (threadIdx.x >> 5)) * rpw;
+  const int64_t r = r0 + (threadIdx.x & 31);
+  if (r0 >= n_rays) return;  // the whole warp
+  const bool live = int(threadIdx.x & 31) < rpw && r < n_rays;
   TrStats ts{0u, 0u, UGP_RAY_OK};
   Ray ray{};
   float t0 = 0.f, t1 = 0.f;
@@ -171,7 +174,7 @@ namespace ugp {
 ugp_status launch_transmittance(const TraceScene& sc, int64_t n, const float* o3, const float* d3,
                                 const float* t0, const float* t1, const int32_t* excl, float* T,
                                 uint8_t* st, cudaStream_t stream) {
-  const unsigned grid = unsigned((n + kTrBlock - 1) / kTrBlock);
+  const unsigned grid = unsigned(tr_grid(n));
   unsigned long long* ctr = trace_counters();
   prof_begin(kStQuery, stream);
   if (ctr)
