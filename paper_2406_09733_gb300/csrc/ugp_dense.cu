@@ -13,7 +13,7 @@
 //      by false-position steps (Illinois rule) and finally by bisection, with F and
 //      F' = 1/2 sum G (Eq. 9) summed across its lanes, and draws the primitive with the
 //      exponential race (smallest E_k / G_k(x_{t_u})) as an argmin across its lanes.
-// A ray whose slot list overflowed, or that has more intervals than a half-warp holds (128), goes
+// A ray whose slot list overflowed, or that has more intervals than a half-warp holds (112), goes
 // to k_dense_big: one warp per ray rebuilds the intervals from the list or by a warp-parallel
 // traversal (up to 32 nodes per step from a shared stack) and solves with 32 lanes. Its intervals
 // (up to kBigCap = 2048) live in a slot of global memory that the warp owns, so the pass is not
@@ -38,7 +38,7 @@ namespace {
 
 constexpr int kDWarps = 4;           // warps per block of the main pass (two rays each)
 constexpr int kHalf = 16;            // lanes of the main pass that finish one ray
-constexpr int kDCap = 128;           // intervals a half-warp of the main pass holds
+constexpr int kDCap = 112;           // intervals a half-warp of the main pass holds (six blocks per SM)
 constexpr int kDStack = 1024;        // traversal stack of a big-pass warp
 constexpr int kDLevels = 8;          // bracket refinements when the intervals do not fit
 constexpr int kDNewton = 64;
@@ -88,14 +88,15 @@ struct Iv {
   float *a, *b, *tn, *ts, *s, *e0, *ex0, *full;
   int* id;  // index with the end-point flags (pack_id)
   int cap;
+  float* amp;  // e0 sqrt(pi) / (4 s), or NULL: formed where it is used
 };
 
 template <int kCap>
 struct Intervals {
-  float a[kCap], b[kCap], tn[kCap], ts[kCap], s[kCap], e0[kCap], ex0[kCap], full[kCap];
+  float a[kCap], b[kCap], tn[kCap], ts[kCap], s[kCap], e0[kCap], ex0[kCap], full[kCap], amp[kCap];
   int id[kCap];
   __device__ Iv view(int off, int cap) {
-    return Iv{a + off, b + off, tn + off, ts + off, s + off, e0 + off, ex0 + off, full + off, id + off, cap};
+    return Iv{a + off, b + off, tn + off, ts + off, s + off, e0 + off, ex0 + off, full + off, id + off, cap, amp + off};
   }
 };
 
@@ -155,7 +156,8 @@ __device__ Finish solve(const Grp<G>& g, const Iv& iv, int n, float lo, float hi
   auto term = [&](int e, float t) {
     if (!(fmaxf(iv.a[e], lo) < t)) return 0.f;
     const float tq = tau_at(t, iv.tn[e], iv.ts[e], iv.s[e]);
-    return iv.e0[e] * (0.25f * kSqrtPi) / iv.s[e] * cut_diff(iv.ex0[e], erfcf(fabsf(tq)), tq);
+    const float amp = iv.amp ? iv.amp[e] : iv.e0[e] * (0.25f * kSqrtPi) / iv.s[e];
+    return amp * cut_diff(iv.ex0[e], erfcf(fabsf(tq)), tq);
   };
   auto evalF = [&](float t, int m, float& f, float& fp) {
     long long fl = 0, fpl = 0;
@@ -294,7 +296,9 @@ __device__ __forceinline__ void collect_one(const Grp<G>& g, const Iv& iv, const
       const float ex0 = tp >= 0.f ? ep : -ep;
       iv.a[i] = hh.a; iv.b[i] = hh.b; iv.tn[i] = hh.tn; iv.ts[i] = hh.ts;
       iv.s[i] = hh.s; iv.e0[i] = hh.e0; iv.ex0[i] = ex0; iv.id[i] = pack_id(hh);
-      iv.full[i] = hh.e0 * (0.25f * kSqrtPi) / hh.s * cut_diff(ex0, erfcf(fabsf(tq)), tq);
+      const float amp = hh.e0 * (0.25f * kSqrtPi) / hh.s;
+      iv.full[i] = amp * cut_diff(ex0, erfcf(fabsf(tq)), tq);
+      if (iv.amp) iv.amp[i] = amp;
     }
   }
   n += __popc(m);
@@ -407,7 +411,11 @@ __device__ __forceinline__ void write_out(const Outputs& O, int idx, const Finis
 // Appends slot j of the table to the list of a bigger pass (counter `count`, array `list`).
 __device__ __forceinline__ void hand_on(int* count, int* list, int j) { list[atomicAdd(count, 1)] = j; }
 
-__global__ void __launch_bounds__(32 * kDWarps) k_dense(TraceScene sc0, DenseQueue q, int64_t n_host,
+// Bound by instruction issue (60% of the slots) and the latency of its dependent steps, so resident
+// warps count: six blocks per SM (80 registers, 112 intervals per ray in shared memory) against five
+// (96, 128) took 2^20 free flights in a 1M-primitive room from 7.27 to 7.06 ms, the stored
+// amplitude of each interval (a division less per term) from 7.32 to 7.27.
+__global__ void __launch_bounds__(32 * kDWarps, 6) k_dense(TraceScene sc0, DenseQueue q, int64_t n_host,
                                                         const int* n_dev, Outputs O) {
   extern __shared__ __align__(16) unsigned char dsm[];
   WarpSmem& W = reinterpret_cast<WarpSmem*>(dsm)[threadIdx.x >> 5];
@@ -458,7 +466,7 @@ __global__ void __launch_bounds__(32 * kDWarps) k_dense(TraceScene sc0, DenseQue
 // block, up to kCap intervals per ray in the warp's slot of q.big_iv; a ray with more has its
 // bracket narrowed by sub-bins (or is handed on to a next pass when `next_count` is given).
 template <int kCap, int kWarps>
-__global__ void __launch_bounds__(32 * kWarps) k_dense_big(TraceScene sc0, DenseQueue q, const int* count_p,
+__global__ void __launch_bounds__(32 * kWarps, 4) k_dense_big(TraceScene sc0, DenseQueue q, const int* count_p,
                                                            const int* __restrict__ list, int* next_count,
                                                            int* __restrict__ next_list, Outputs O) {
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -468,7 +476,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_dense_big(TraceScene sc0, Dense
   // this warp's interval slot (the grid has at most q.big_slots warps)
   float* slot = q.big_iv + size_t(blockIdx.x * kWarps + (threadIdx.x >> 5)) * (size_t(kCap) * 9);
   const Iv iv{slot, slot + kCap, slot + 2 * kCap, slot + 3 * kCap, slot + 4 * kCap, slot + 5 * kCap,
-              slot + 6 * kCap, slot + 7 * kCap, reinterpret_cast<int*>(slot + 8 * kCap), kCap};
+              slot + 6 * kCap, slot + 7 * kCap, reinterpret_cast<int*>(slot + 8 * kCap), kCap, nullptr};
   const int count = *reinterpret_cast<const volatile int*>(count_p);
   for (int h = blockIdx.x * kWarps + (threadIdx.x >> 5); h < count; h += gridDim.x * kWarps) {
     const int j = list[h];
