@@ -312,7 +312,7 @@ __global__ void k_collapse4(int n_int, const float4* __restrict__ nodes, const i
   uint32_t qlo[3] = {0u, 0u, 0u}, qhi[3] = {0u, 0u, 0u}, ex = 0u;
   for (int a = 0; a < 3; ++a) {
     // a power-of-two spacing 2^e >= extent / 254 (frexp: extent / 254 = f 2^e, f in [1/2, 1));
-    // the spare step absorbs the rounding of o + q 2^e
+    // the spare step absorbs the margins and the rounding of o + q 2^e
     const float ext = hi[a] - lo[a];
     int e = -126;
     if (ext > 0.f) {
@@ -320,9 +320,13 @@ __global__ void k_collapse4(int n_int, const float4* __restrict__ nodes, const i
       e = max(-126, min(e, 126));
     }
     const float sp = ldexpf(1.f, e), isp = ldexpf(1.f, -e);
+    // the faces keep a margin of 2^-7 grid steps to the boxes (the rounding of the node test); the
+    // grid starts 2^-5 steps below the union so that its lowest face has one as well
+    constexpr float kMargin = 0.0078125f;
+    lo[a] -= 4.f * kMargin * sp;
     for (int c = 0; c < m; ++c) {
-      int ql = int(floorf((box[c][a] - lo[a]) * isp));
-      int qh = int(ceilf((box[c][3 + a] - lo[a]) * isp));
+      int ql = int(floorf((box[c][a] - lo[a]) * isp - kMargin));
+      int qh = int(ceilf((box[c][3 + a] - lo[a]) * isp + kMargin));
       ql = max(0, min(ql, 255));
       qh = max(0, min(qh, 255));
       while (ql > 0 && fmaf(float(ql), sp, lo[a]) > box[c][a]) --ql;
