@@ -60,14 +60,21 @@ __device__ __forceinline__ float4 ld4(const float* p, int64_t i) {
 // Bounding box of the k-ellipsoid x = mu + k R S v, |v| = 1: half extent along axis i is
 // k * sqrt(sum_j (R_ij s_j)^2).  Widened by a few float32 ulps so the box stays
 // conservative for the float32 interval test.
-__global__ void k_prim_bounds(int64_t n, const float* __restrict__ mean3, const float* __restrict__ quat4,
-                              const float* __restrict__ scale3, const float* __restrict__ mag, float k,
-                              float4* __restrict__ aabb, int* __restrict__ bounds,
-                              unsigned long long* __restrict__ n_invalid) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  float cx = 0.f, cy = 0.f, cz = 0.f;
-  bool has = false;
-  if (i < n) {
+//
+// The bounds of the means are reduced per thread, then per block, over a grid of resident blocks: one
+// atomic per bound and block. One per warp of primitives (172,000 of them at 5.5M, on six
+// addresses) took 0.68 ms, against 0.08 for the arrays themselves.
+constexpr int kBoundsBlocks = 152 * 8;
+__global__ void __launch_bounds__(256) k_prim_bounds(int64_t n, const float* __restrict__ mean3,
+                                                     const float* __restrict__ quat4, const float* __restrict__ scale3,
+                                                     const float* __restrict__ mag, float k, float4* __restrict__ aabb,
+                                                     int* __restrict__ bounds,
+                                                     unsigned long long* __restrict__ n_invalid) {
+  __shared__ int red[6][8];
+  const float big = 3.0e38f;
+  float v[6] = {big, big, big, big, big, big};  // min of the means and of their negatives
+  unsigned bad = 0u;
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
     const float3 m = ld3(mean3, i);
     const float4 q = ld4(quat4, i);
     const float3 s = ld3(scale3, i);
@@ -83,24 +90,29 @@ __global__ void k_prim_bounds(int64_t n, const float* __restrict__ mean3, const 
       }
       aabb[2 * i] = make_float4(m.x - e[0], m.y - e[1], m.z - e[2], 0.f);
       aabb[2 * i + 1] = make_float4(m.x + e[0], m.y + e[1], m.z + e[2], 0.f);
-      cx = m.x; cy = m.y; cz = m.z;
-      has = true;
+      for (int r = 0; r < 3; ++r) {
+        v[r] = fminf(v[r], mm[r]);
+        v[3 + r] = fminf(v[3 + r], -mm[r]);
+      }
     } else {
       // An invalid primitive keeps a point box; its record is flagged and never hit.
       const float x = isfinite(m.x) ? m.x : 0.f, y = isfinite(m.y) ? m.y : 0.f,
                   z = isfinite(m.z) ? m.z : 0.f;
       aabb[2 * i] = make_float4(x, y, z, 0.f);
       aabb[2 * i + 1] = make_float4(x, y, z, 0.f);
-      atomicAdd(n_invalid, 1ull);
+      ++bad;
     }
   }
-  // Centroid bounds: warp min-reduction of the ordered-int encodings, one atomic per warp.
-  const float big = 3.0e38f;
-  const float v[6] = {has ? cx : big, has ? cy : big, has ? cz : big,
-                      has ? -cx : big, has ? -cy : big, has ? -cz : big};
+  if (bad) atomicAdd(n_invalid, (unsigned long long)bad);
   for (int a = 0; a < 6; ++a) {
     const int r = __reduce_min_sync(0xffffffffu, f2o(v[a]));
-    if ((threadIdx.x & 31) == 0) atomicMin(&bounds[a], r);
+    if ((threadIdx.x & 31) == 0) red[a][threadIdx.x >> 5] = r;
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    int r = red[threadIdx.x][0];
+    for (int w = 1; w < 8; ++w) r = min(r, red[threadIdx.x][w]);
+    atomicMin(&bounds[threadIdx.x], r);
   }
 }
 
@@ -468,7 +480,7 @@ extern "C" ugp_status ugp_build_bvh(const ugp_prims* prims, float cutoff_eps, vo
   prof_begin(kStBuild, st);
   UGP_CUDA_CHECK(cudaMemsetAsync(ws + L.bounds, 0, 64, st));
   k_init_bounds<<<1, 32, 0, st>>>(bounds, nullptr);
-  k_prim_bounds<<<G, T, 0, st>>>(n, prims->mean3, prims->quat4, prims->scale3, prims->magnitude, b->k,
+  k_prim_bounds<<<G < unsigned(kBoundsBlocks) ? G : unsigned(kBoundsBlocks), T, 0, st>>>(n, prims->mean3, prims->quat4, prims->scale3, prims->magnitude, b->k,
                                  aabb, bounds, n_invalid);
   UGP_CUDA_CHECK(cudaGetLastError());
   int4* nodes_i = reinterpret_cast<int4*>(ws + L.nodes);
