@@ -29,9 +29,9 @@ constexpr int kNodeF4 = 4;
 // Child reference of the unused second child of a one-primitive tree's root.
 constexpr int kEmptyChild = INT32_MIN;
 
-// Device layout of one 4-wide node (64 B) of the collapsed tree the hot traversals walk: the
-// binary internal nodes at even depth, each with the (up to four) children and grandchildren
-// below it, their boxes quantised to 8 bits per face against a per-node grid.
+// Device layout of one 4-wide node (64 B) of the collapsed tree the hot traversals walk: a binary
+// internal node with up to four of its descendants (its children, the largest internal one replaced
+// by its own two until there are four), their boxes quantised to 8 bits per face against a per-node grid.
 //   w0 = (o.x, o.y, o.z as float bits, exponents: byte a = e_a + 128 for axes a = 0, 1, 2)
 //   w1 = (lo_x, lo_y, lo_z, hi_x)  byte c of each word: child c's quantised face
 //   w2 = (hi_y, hi_z, 0, 0)
@@ -41,7 +41,7 @@ constexpr int kEmptyChild = INT32_MIN;
 // outwards with a margin of 2^-7 grid steps, so the quantised box contains the exact one by more than
 // the node test's rounding. An empty slot's box is inverted
 // (lo = 255, hi = 0 on every axis), so no ray enters it. A 4-wide node sits at the index of its
-// binary node (the array has holes at odd depths, which are never read).
+// binary node (the nodes that were absorbed are never read).
 constexpr int kNode4U4 = 4;
 
 }  // namespace ugp
