@@ -54,7 +54,7 @@ struct ugp_bvh {
   float k;
   float k2;
   const float4* nodes;
-  const uint4* nodes4;       // the 4-wide quantised tree (same indices as nodes, even depths only)
+  const uint4* nodes4;       // the 4-wide quantised tree (same indices as nodes)
   const float4* prims;
   const float4* wlo;         // low float parts of W, 3 float4 per leaf slot
   const float* bounds_dev;   // in the workspace: ordered-int centroid bounds, root box, invalid count

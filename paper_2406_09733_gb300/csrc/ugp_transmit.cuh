@@ -1,4 +1,5 @@
-// Transmittance (Sec. 5.3, Eq. 7) of one ray: device code shared by the query and the renderer.
+// Traversal of all primitives along a ray with pooled leaf steps, and the transmittance (Sec. 5.3,
+// Eq. 7) of one ray by it: device code shared by the queries, the renderer and the batch server.
 #pragma once
 
 #include "ugp_gauss.cuh"
@@ -13,34 +14,34 @@ struct TrStats {
 
 constexpr int kTrLeafQ = 10;  // primitives a lane may hold back (top of its stack column)
 
-// Returns tau = 1/2 sum_k I_k(clip_k) over [t0, t1], stopping once it reaches 1 (then T = 0).
-// The sum is kept in 64-bit fixed point (units of 2^-40), so it is the same in any traversal
-// order and whichever lanes test a ray's primitives (terms below 2^-41 are dropped: under 1e-10
-// in tau for a few hundred of them); nearest-child-first only makes the early exit come sooner.
-// `stk` points at this thread's column of a shared-memory stack with `stride` between levels,
-// `acc` at this thread's entry of a shared array of sums and `owner` at its entry of a shared
-// int array (its neighbours in the warp are the other lanes' entries). The whole warp calls
-// together (lanes without a ray pass live = false) and runs in steps: a node
+// Visits every primitive whose clipped interval over [t0, t1] may meet [t0, t_far] (t_far <= t1).
+// `stk` points at this thread's column of a shared-memory stack with `stride` between levels and
+// `owner` at its entry of a shared int array (its neighbours in the warp are the other lanes' entries).
+// The whole warp calls together (lanes without a ray pass live = false) and runs in steps: a node
 // step visits one node per lane and holds back the primitives it meets (up to kTrLeafQ, kept at
 // the top of the stack column); a leaf step, taken once the lanes hold a primitive for each of
 // them (or a queue is nearly full or a traversal is over), spreads the held-back primitives over
-// the lanes, one per lane whichever ray it belongs to, and each lane adds its primitive's term to
-// the owner's sum with a shared-memory atomic. The kernel is bound by instruction issue (ALU pipe):
-// one packed warp sum per step instead of six votes, one erf for an interval whose two ends are the
-// ellipsoid's, and the shared recomputation of ill-conditioned hits took 1,000,003 light-sample rays in
-// a 1M-primitive room from 3.42 to 3.04 ms.
+// the lanes, one per lane whichever ray it belongs to. The kernels are bound by instruction issue (ALU
+// pipe): one packed warp sum per step instead of six votes, one erf for an interval whose two ends are
+// the ellipsoid's, and the shared recomputation of ill-conditioned hits took 1,000,003 light-sample rays
+// in a 1M-primitive room from 3.42 to 3.04 ms.
+//
+// `P` collects the hits:
+//   leaf(bool ok, const PrimHit& h, int o, bool work, int off, int mine)   called by all lanes in a leaf
+//       step: this lane's primitive is hit (ok) by the ray of lane o; `work` lanes took a primitive, those
+//       of one ray are neighbours; this lane's own ray's start at lane off, `mine` of them were waiting
+//   bool enough()    after it, by lanes whose primitives were taken: nothing more can matter
+//   kNearFirst       children are visited nearest first
 static_assert(kTrLeafQ < 16, "queue lengths are summed from four bit planes");
-static __device__ float tr_optical_depth(const TraceScene& sc, const Ray& ray, float t0, float t1, int ex,
-                                         int* stk, int stride, unsigned long long* acc, int* owner, TrStats& ts,
-                                         bool live) {
+template <class P>
+static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& ray, float t0, float t1, float t_far,
+                                               int ex, int* stk, int stride, int* owner, TrStats& ts, bool live,
+                                               P& pol) {
   constexpr unsigned mask = 0xffffffffu;
   const int lane = int(threadIdx.x) & 31;
   const unsigned below_me = (1u << lane) - 1u;
-  constexpr float kScale = 1099511627776.f;  // 2^40
-  constexpr unsigned long long kOne = 1ull << 40;
-  *acc = 0ull;
   int sp = 0, node = 0, nq = 0;
-  bool tdone = !(live && sc.n_prims > 0 && t0 < t1), done = tdone;
+  bool tdone = !(live && sc.n_prims > 0 && t0 < t_far), done = tdone;
   int* lq = stk + (kTrStack - kTrLeafQ) * stride;
   __syncwarp(mask);
   for (;;) {
@@ -81,13 +82,12 @@ static __device__ float tr_optical_depth(const TraceScene& sc, const Ray& ray, f
       const float k2 = __shfl_sync(mask, sc.k2, o);
       PrimHit h;
       const int slot = work ? lq[(nq_o - 1 - (lane - off_o)) * stride + (o - lane)] : 0;
-      if (prim_test_of<true>(work, prims, wlo, slot, ro, t0o, t1o, k2, exo, h))
-        atomicAdd(acc + (o - lane),
-                  (unsigned long long)__float2ll_rn(fminf(fmaxf(hit_half_integral(h), 0.f), 2.f) * kScale));
+      const bool ok = prim_test_of<true>(work, prims, wlo, slot, ro, t0o, t1o, k2, exo, h);
+      pol.leaf(ok, h, o, work, off, mine);
       __syncwarp(mask);
       if (mine > 0) {
         nq = mine - min(mine, max(0, 32 - off));
-        if (*acc >= kOne) {  // saturated: T = 0 whatever follows
+        if (pol.enough()) {
           done = true;
           nq = 0;
         }
@@ -100,7 +100,7 @@ static __device__ float tr_optical_depth(const TraceScene& sc, const Ray& ray, f
       } else {
         float en[4];
         int ch[4];
-        const unsigned hm = node4_test(sc.nodes4, node, ray, t0, t1, en, ch);
+        const unsigned hm = node4_test(sc.nodes4, node, ray, t0, t_far, en, ch);
         ++ts.n_nodes;
         float tk[4];
         int rk[4];
@@ -127,7 +127,7 @@ static __device__ float tr_optical_depth(const TraceScene& sc, const Ray& ray, f
             ++nk;
           }
         }
-        sort4(tk, rk);
+        if (P::kNearFirst || rk[0] < 0) sort4(tk, rk);  // at least, the first is one that was hit
         if (bad) {
           ts.st = UGP_RAY_BAD_NODE;
           tdone = true;
@@ -156,8 +156,34 @@ static __device__ float tr_optical_depth(const TraceScene& sc, const Ray& ray, f
     }
     if (tdone && nq == 0) done = true;
   }
+}
+
+// Returns tau = 1/2 sum_k I_k(clip_k) over [t0, t1], stopping once it reaches 1 (then T = 0).
+// The sum is kept in 64-bit fixed point (units of 2^-40), so it is the same in any traversal
+// order and whichever lanes test a ray's primitives (terms below 2^-41 are dropped: under 1e-10
+// in tau for a few hundred of them); nearest-child-first only makes the early exit come sooner.
+// `acc` points at this thread's entry of a shared array of sums; each lane of a leaf step adds its
+// primitive's term to the owner's with a shared-memory atomic. Other arguments as for tr_walk.
+struct DepthSum {
+  static constexpr bool kNearFirst = true;
+  static constexpr float kScale = 1099511627776.f;  // 2^40
+  static constexpr unsigned long long kOne = 1ull << 40;
+  unsigned long long* acc;
+  __device__ void leaf(bool ok, const PrimHit& h, int o, bool, int, int) {
+    if (ok)
+      atomicAdd(acc + (o - (int(threadIdx.x) & 31)),
+                (unsigned long long)__float2ll_rn(fminf(fmaxf(hit_half_integral(h), 0.f), 2.f) * kScale));
+  }
+  __device__ bool enough() const { return *acc >= kOne; }  // saturated: T = 0 whatever follows
+};
+static __device__ float tr_optical_depth(const TraceScene& sc, const Ray& ray, float t0, float t1, int ex,
+                                         int* stk, int stride, unsigned long long* acc, int* owner, TrStats& ts,
+                                         bool live) {
+  DepthSum pol{acc};
+  *acc = 0ull;
+  tr_walk(sc, ray, t0, t1, t1, ex, stk, stride, owner, ts, live, pol);
   const unsigned long long a = *acc;
-  return a >= kOne ? 1.f : float(a) * (1.f / kScale);
+  return a >= DepthSum::kOne ? 1.f : float(a) * (1.f / DepthSum::kScale);
 }
 
 }  // namespace ugp
