@@ -117,22 +117,9 @@ struct ArraySrc {
 
 struct ArrayDst {
   float *head, *mix;
-  GuideCfgDev cfg;
-  // the mixture when asked for (then a head asked for as well is written here, per thread),
-  // else the head
-  __device__ float* row_out(int64_t r) const { return (mix ? mix : head) + kGOut * r; }
-  __device__ void values(int64_t r, const float (&Y)[kGOut], float (&out)[kGOut]) const {
-    if (mix) {
-      if (head) {
-#pragma unroll
-        for (int j = 0; j < kGOut; ++j) head[kGOut * r + j] = Y[j];
-      }
-      mixture_from_head(cfg, Y, out);
-    } else {
-#pragma unroll
-      for (int j = 0; j < kGOut; ++j) out[j] = Y[j];
-    }
-  }
+  __device__ bool head_rows() const { return head != nullptr; }
+  __device__ bool mix_rows() const { return mix != nullptr; }
+  __device__ float* row_out(int which, int64_t r) const { return (which ? mix : head) + kGOut * r; }
 };
 
 int elementwise_grid(int64_t n, int block) {
@@ -199,7 +186,7 @@ extern "C" ugp_status ugp_guide_forward(const ugp_guide* g, int64_t n, const flo
   if ((s = launch_guide_pack(g->params, ws.img, st)) != UGP_OK) return s;
   const GuideDev gd{guide_cfg_dev(g), ws.img, ws.err};
   prof_begin(kStGuide, st);
-  s = launch_guide_forward(gd, ArraySrc{x3, wo3, nullptr, nullptr}, ArrayDst{head_out, mix_out, gd.cfg}, n, nullptr,
+  s = launch_guide_forward(gd, ArraySrc{x3, wo3, nullptr, nullptr}, ArrayDst{head_out, mix_out}, n, nullptr,
                            n, st);
   prof_end(kStGuide, st);
   return s;

@@ -106,7 +106,7 @@ __device__ __forceinline__ float vmf_log_norm(float k) {
   return logf(k) - 1.83787706640934548f - logf(-expm1f(-2.f * k));
 }
 
-// Mixture (per lobe mu (3), kappa, pi) from the 40 head outputs.
+// Mixture (per lobe mu (3), kappa, pi) from the 40 head outputs (may be in place).
 __device__ __forceinline__ void mixture_from_head(const GuideCfgDev& c, const float Y[kGOut], float mix[kGOut]) {
   float amax = -3.4e38f;
 #pragma unroll
@@ -117,14 +117,14 @@ __device__ __forceinline__ void mixture_from_head(const GuideCfgDev& c, const fl
   const float iz = 1.f / z;
 #pragma unroll
   for (int j = 0; j < kGLobes; ++j) {
-    const float mx = Y[5 * j], my = Y[5 * j + 1], mz = Y[5 * j + 2];
+    const float mx = Y[5 * j], my = Y[5 * j + 1], mz = Y[5 * j + 2], s = Y[5 * j + 3], a = Y[5 * j + 4];
     const float n = sqrtf(mx * mx + my * my + mz * mz);
     const float in = n > 0.f ? 1.f / n : 0.f;
     mix[5 * j] = n > 0.f ? mx * in : 0.f;
     mix[5 * j + 1] = n > 0.f ? my * in : 0.f;
     mix[5 * j + 2] = n > 0.f ? mz * in : 1.f;
-    mix[5 * j + 3] = fminf(c.kappa_max, c.kappa_min + softplusf(Y[5 * j + 3]));
-    mix[5 * j + 4] = expf(Y[5 * j + 4] - amax) * iz;
+    mix[5 * j + 3] = fminf(c.kappa_max, c.kappa_min + softplusf(s));
+    mix[5 * j + 4] = expf(a - amax) * iz;
   }
 }
 

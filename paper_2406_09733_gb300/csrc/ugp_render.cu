@@ -401,11 +401,9 @@ struct ShadeQueueSrc {
 struct MixByPathDst {
   const int* q;
   float* mix;
-  GuideCfgDev cfg;
-  __device__ float* row_out(int64_t r) const { return mix + size_t(q[r]) * kGOut; }
-  __device__ void values(int64_t, const float (&Y)[kGOut], float (&out)[kGOut]) const {
-    mixture_from_head(cfg, Y, out);
-  }
+  __device__ bool head_rows() const { return false; }
+  __device__ bool mix_rows() const { return true; }
+  __device__ float* row_out(int, int64_t r) const { return mix + size_t(q[r]) * kGOut; }
 };
 
 // Training rows: selected log entries, taken cyclically from `offset` (n_sel entries).
@@ -667,7 +665,7 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
         prof_begin(kStGuide, st);
         const ugp_status gsx = launch_guide_forward(
             gd, ShadeQueueSrc{ps, queue[cur], md.type, b, params->max_depth},
-            MixByPathDst{queue[cur], const_cast<float*>(gs.mix), gd.cfg}, n, counts + cur, n, st);
+            MixByPathDst{queue[cur], const_cast<float*>(gs.mix)}, n, counts + cur, n, st);
         prof_end(kStGuide, st);
         if (gsx != UGP_OK) return gsx;
       }
