@@ -327,6 +327,7 @@ __global__ void __launch_bounds__(128) k_b_shade(BState S) {
   }
 }
 
+template <bool kFew>
 __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_b_shadow(BState S) {
   __shared__ int stk[kTrStack * kTrBlock];
   __shared__ unsigned long long tr_acc[kTrBlock];
@@ -335,10 +336,12 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_b_shadow(BState S)
   const BPaths& P = S.P;
   // one ray per thread over a grid sized for the pool (fewer per warp when there are few):
   // the hardware spreads the blocks
-  const int rpw = rays_per_warp(count, min(int(gridDim.x) * (kTrBlock / 32), kTrWarps));
-  const int j0 = int(blockIdx.x * (kTrBlock / 32) + (threadIdx.x >> 5)) * rpw, j = j0 + int(threadIdx.x & 31);
+  // (kFew: a group of lanes each)
+  const int lg = kFew ? tr_group(count) : 0, lane = int(threadIdx.x & 31);
+  const int rpw = kFew ? 32 >> lg : rays_per_warp(count, min(int(gridDim.x) * (kTrBlock / 32), kTrWarps));
+  const int j0 = int(blockIdx.x * (kTrBlock / 32) + (threadIdx.x >> 5)) * rpw, j = j0 + (lane >> lg);
   if (j0 >= count) return;  // the whole warp
-  const bool live = int(threadIdx.x & 31) < rpw && j < count;
+  const bool live = (lane >> lg) < rpw && j < count;
   TrStats ts{0u, 0u, UGP_RAY_OK};
   TraceScene sc{};
   Ray ray{};
@@ -351,9 +354,9 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_b_shadow(BState S)
     dist = S.sh.dist[j];
     ex = S.sh.excl[j];
   }
-  const float tau = tr_optical_depth(sc, ray, 0.f, dist, ex, stk + threadIdx.x, kTrBlock, tr_acc + threadIdx.x,
-                                     tr_owner + threadIdx.x, ts, live);
-  if (!live) return;
+  const float tau = tr_optical_depth<kFew>(sc, ray, 0.f, dist, ex, stk + threadIdx.x, kTrBlock, tr_acc + threadIdx.x,
+                                           tr_owner + threadIdx.x, ts, live, lg);
+  if (!live || (lane & ((1 << lg) - 1)) != 0) return;
   const float T = fmaxf(0.f, 1.f - tau);
   if (T > 0.f) {
     P.ps.lr[p] += T * S.sh.cr[j];
@@ -491,12 +494,13 @@ int grid_of(const void* kernel, int block, int64_t n) {
 // Persistent grid sizes of the wave kernels for a pool (computed before any stream capture).
 struct WaveGrids {
   int regen, ext, shade, shadow, retire;
+  bool few;  // shadow rays in groups of lanes
 };
 WaveGrids wave_grids(int64_t pool) {
   const int ext_need = int((pool + kFFBlock / 32 - 1) / (kFFBlock / 32)), ext_cap = scan_grid((const void*)k_b_extend);
   return WaveGrids{grid_of((const void*)k_b_regen, 256, pool), ext_need < ext_cap ? ext_need : ext_cap,
-                   grid_of((const void*)k_b_shade, 128, pool), tr_grid(pool),
-                   grid_of((const void*)k_b_retire, 256, pool)};
+                   grid_of((const void*)k_b_shade, 128, pool), pool <= kTrFew ? tr_few_grid(pool) : tr_grid(pool),
+                   grid_of((const void*)k_b_retire, 256, pool), pool <= kTrFew};
 }
 
 // Launches one wave on `st` (also used while capturing the graph body).
@@ -510,7 +514,7 @@ ugp_status launch_wave(const BState& S, const WaveGrids& g, cudaGraphConditional
                               nullptr, 0, nullptr, &S.ctl->dense_err, st);
   if (s != UGP_OK) return s;
   k_b_shade<<<g.shade, 128, 0, st>>>(S);
-  k_b_shadow<<<g.shadow, kTrBlock, 0, st>>>(S);
+  (g.few ? k_b_shadow<true> : k_b_shadow<false>)<<<g.shadow, kTrBlock, 0, st>>>(S);
   k_b_retire<<<g.retire, 256, 0, st>>>(S);
   k_b_cond<<<1, 32, 0, st>>>(S, h, use_graph);
   UGP_CUDA_CHECK(cudaGetLastError());

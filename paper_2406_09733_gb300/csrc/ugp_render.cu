@@ -329,6 +329,7 @@ __global__ void __launch_bounds__(128) k_shade(MatDev mats, LightsDev L, uint2 k
   }
 }
 
+template <bool kFew>
 __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_shadow(TraceScene sc, ShadowSoA sh, const int* cnt, PathSoA ps,
                                                      unsigned long long* rays, unsigned long long* stats) {
   __shared__ int stk[kTrStack * kTrBlock];
@@ -338,10 +339,12 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_shadow(TraceScene 
   if (blockIdx.x == 0 && threadIdx.x == 0 && rays) atomicAdd(rays + 1, (unsigned long long)count);
   // one ray per thread over a grid sized for the longest queue (fewer per warp when there are
   // few): the hardware spreads the blocks
-  const int rpw = rays_per_warp(count, min(int(gridDim.x) * (kTrBlock / 32), kTrWarps));
-  const int j0 = int(blockIdx.x * (kTrBlock / 32) + (threadIdx.x >> 5)) * rpw, j = j0 + int(threadIdx.x & 31);
+  // (kFew: a group of lanes each)
+  const int lg = kFew ? tr_group(count) : 0, lane = int(threadIdx.x & 31);
+  const int rpw = kFew ? 32 >> lg : rays_per_warp(count, min(int(gridDim.x) * (kTrBlock / 32), kTrWarps));
+  const int j0 = int(blockIdx.x * (kTrBlock / 32) + (threadIdx.x >> 5)) * rpw, j = j0 + (lane >> lg);
   if (j0 >= count) return;  // the whole warp
-  const bool live = int(threadIdx.x & 31) < rpw && j < count;
+  const bool live = (lane >> lg) < rpw && j < count;
   TrStats ts{0u, 0u, UGP_RAY_OK};
   Ray ray{};
   float dist = 0.f;
@@ -353,9 +356,9 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_shadow(TraceScene 
   }
   // a negative distance marks a light sample of an emissive primitive: it counts when the
   // point lies before saturation (T > 0) and is not scaled by T
-  const float tau = tr_optical_depth(sc, ray, 0.f, fabsf(dist), ex, stk + threadIdx.x, kTrBlock,
-                                     tr_acc + threadIdx.x, tr_owner + threadIdx.x, ts, live);
-  if (!live) return;
+  const float tau = tr_optical_depth<kFew>(sc, ray, 0.f, fabsf(dist), ex, stk + threadIdx.x, kTrBlock,
+                                           tr_acc + threadIdx.x, tr_owner + threadIdx.x, ts, live, lg);
+  if (!live || (lane & ((1 << lg) - 1)) != 0) return;
   const float T = fmaxf(0.f, 1.f - tau);
   if (T > 0.f) {
     const float s = dist < 0.f ? 1.f : T;
@@ -642,7 +645,10 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
   const int g_cam = grid_for((const void*)k_camera, 256, n);
   const int g_ext = grid_for((const void*)k_extend, kFFBlock, 32 * n);  // down to one ray per warp
   const int g_shade = guide ? grid_for((const void*)k_shade<true>, 128, n) : grid_for((const void*)k_shade<false>, 128, n);
-  const int g_shadow = tr_grid(n);
+  // small images: groups of lanes per ray (the statistics count whole rays per lane)
+  const bool few = n <= kTrFew && !stats;
+  const int g_shadow = few ? tr_few_grid(n) : tr_grid(n);
+  const auto shadow = few ? k_shadow<true> : k_shadow<false>;
   const int g_acc = grid_for((const void*)k_accumulate, 256, n);
   for (int si = 0; si < params->spp; ++si) {
     const int sample = params->spp_begin + si;
@@ -683,12 +689,12 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
       // this order, so the sum does not depend on scheduling
       if (params->nee && Ld.has_quad) {
         prof_begin(kStShadow, st);
-        k_shadow<<<g_shadow, kTrBlock, 0, st>>>(sc, sh, counts + 2, ps, ray_counts, stats);
+        shadow<<<g_shadow, kTrBlock, 0, st>>>(sc, sh, counts + 2, ps, ray_counts, stats);
         prof_end(kStShadow, st);
       }
       if (Em.cdf) {
         prof_begin(kStShadow, st);
-        k_shadow<<<g_shadow, kTrBlock, 0, st>>>(sc, she, counts + 4, ps, ray_counts, stats);
+        shadow<<<g_shadow, kTrBlock, 0, st>>>(sc, she, counts + 4, ps, ray_counts, stats);
         prof_end(kStShadow, st);
       }
       cur = nxt;

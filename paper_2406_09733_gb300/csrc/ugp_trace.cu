@@ -43,6 +43,35 @@ k_transmittance(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, con
   if (STATS) add_counters(ctr, ts.n_nodes, ts.n_prims, 1u, 1u, 0u);
 }
 
+// The same for few rays, a group of lanes per ray.
+__global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM)
+k_transmittance_few(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, const float* __restrict__ d3,
+                    const float* __restrict__ t0a, const float* __restrict__ t1a, const int32_t* __restrict__ excl,
+                    float* __restrict__ T_out, uint8_t* __restrict__ st_out) {
+  __shared__ int stk[kTrStack * kTrBlock];
+  __shared__ unsigned long long tr_acc[kTrBlock];
+  __shared__ int tr_owner[kTrBlock];
+  const int lg = tr_group(n_rays);
+  const int64_t r = (int64_t(blockIdx.x) * kTrBlock + threadIdx.x) >> lg;
+  if ((int64_t(blockIdx.x) * kTrBlock + (threadIdx.x & ~31)) >> lg >= n_rays) return;  // the whole warp
+  const bool live = r < n_rays;
+  TrStats ts{0u, 0u, UGP_RAY_OK};
+  Ray ray{};
+  float t0 = 0.f, t1 = 0.f;
+  int ex = -1;
+  if (live) {
+    ray = make_ray(ld3(o3, r), ld3(d3, r));
+    t0 = __ldg(t0a + r);
+    t1 = __ldg(t1a + r);
+    if (excl) ex = __ldg(excl + r);
+  }
+  const float acc = tr_optical_depth<true>(sc, ray, t0, t1, ex, stk + threadIdx.x, kTrBlock, tr_acc + threadIdx.x,
+                                           tr_owner + threadIdx.x, ts, live, lg);
+  if (!live || (threadIdx.x & ((1 << lg) - 1)) != 0) return;
+  T_out[r] = fmaxf(0.f, 1.f - acc);
+  if (st_out) st_out[r] = ts.st;
+}
+
 // All hits along each ray, for hit-set diagnostics (no early exit).
 __global__ void __launch_bounds__(kTrBlock)
 k_collect_hits(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, const float* __restrict__ d3,
@@ -177,10 +206,13 @@ ugp_status launch_transmittance(const TraceScene& sc, int64_t n, const float* o3
   const unsigned grid = unsigned(tr_grid(n));
   unsigned long long* ctr = trace_counters();
   prof_begin(kStQuery, stream);
-  if (ctr)
+  if (ctr) {
     k_transmittance<true><<<grid, kTrBlock, 0, stream>>>(sc, n, o3, d3, t0, t1, excl, T, st, ctr);
-  else
+  } else if (n <= kTrFew) {
+    k_transmittance_few<<<tr_few_grid(n), kTrBlock, 0, stream>>>(sc, n, o3, d3, t0, t1, excl, T, st);
+  } else {
     k_transmittance<false><<<grid, kTrBlock, 0, stream>>>(sc, n, o3, d3, t0, t1, excl, T, st, ctr);
+  }
   prof_end(kStQuery, stream);
   UGP_CUDA_CHECK(cudaGetLastError());
   return UGP_OK;

@@ -35,6 +35,29 @@ struct TraceScene {
   float k2;
 };
 
+// Launches of few rays give each ray a group of lanes (tr_walk): log2 of its size for n rays, 0 for
+// a lane each. Light-sample rays of a 1M-primitive room, us, by lanes per ray:
+//   rays      1     2     4     8    16    32
+//     2K    169   152    88    56    39    31
+//     8K    225   174    98    66    57    63
+//    16K    269   190   115    80    89   105
+//    30K    347   213   167   143   151   186
+//    60K    406   279   242   233   262   342
+//   120K    493   468   425   434   505   667
+//   250K    848   830   793   849  1009  1368
+//   500K   1494  1527  1515  1647  1987  2717
+constexpr int kTrFew = 72 * kTrWarps;
+__host__ __device__ constexpr int tr_group(int64_t n) {
+  return n <= kTrWarps ? 5 : (2 * n <= 5 * kTrWarps ? 4 : (n <= 16 * kTrWarps ? 3 : (n <= kTrFew ? 2 : 0)));
+}
+// Blocks of a launch of up to n <= kTrFew rays in groups.
+inline int tr_few_grid(int64_t n) {
+  int64_t t = n << tr_group(n);  // lanes; a smaller count may take more of them
+  for (const int64_t b : {int64_t(kTrWarps), int64_t(5) * kTrWarps / 2, int64_t(16) * kTrWarps})
+    if (b < n && b << tr_group(b) > t) t = b << tr_group(b);
+  return int((t + kTrBlock - 1) / kTrBlock);
+}
+
 // Blocks of a transmittance launch of up to n rays.
 inline int tr_grid(int64_t n) {
   const int64_t full = (n + kTrBlock - 1) / kTrBlock;

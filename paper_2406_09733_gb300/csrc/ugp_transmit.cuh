@@ -33,16 +33,31 @@ constexpr int kTrLeafQ = 10;  // primitives a lane may hold back (top of its sta
 //   bool enough()    after it, by lanes whose primitives were taken: nothing more can matter
 //   kNearFirst       children are visited nearest first
 static_assert(kTrLeafQ < 16, "queue lengths are summed from four bit planes");
-template <class P>
+//
+// With kGroup, 1 << lg neighbouring lanes share a ray (its arguments are the same on all of them): the
+// stack columns of a group are one stack, and a node step takes a node per lane from its top, nearest in
+// the group's first lane. A launch of few rays is bound by the chain of dependent steps of its longest
+// ray, and this shortens the chain, where spreading the rays over the warps left most lanes idle (figures at
+// tr_group).
+template <bool kGroup, class P>
 static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& ray, float t0, float t1, float t_far,
                                                int ex, int* stk, int stride, int* owner, TrStats& ts, bool live,
-                                               P& pol) {
+                                               int lg, P& pol) {
   constexpr unsigned mask = 0xffffffffu;
   const int lane = int(threadIdx.x) & 31;
   const unsigned below_me = (1u << lane) - 1u;
   int sp = 0, node = 0, nq = 0;
   bool tdone = !(live && sc.n_prims > 0 && t0 < t_far), done = tdone;
   int* lq = stk + (kTrStack - kTrLeafQ) * stride;
+  // the group: its first lane, its lanes, its stack (entry i in row i >> lg of column i & (lanes - 1))
+  const int gsize = kGroup ? 1 << lg : 1, gbase = lane & ~(gsize - 1);
+  const unsigned glanes = (gsize == 32 ? ~0u : (1u << gsize) - 1u) << gbase;
+  int* const gstk = stk - (lane - gbase);
+  auto at = [&](int i) -> int& { return gstk[(i >> lg) * stride + (i & (gsize - 1))]; };
+  if (kGroup) {
+    if (lane == gbase) at(0) = 0;
+    sp = 1;  // entries of the group's stack (with a lane per ray: below the current node)
+  }
   __syncwarp(mask);
   for (;;) {
     // one packed sum: held-back primitives (9 bits), lanes at work, lanes that need a leaf step (a
@@ -85,13 +100,67 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
       const bool ok = prim_test_of<true>(work, prims, wlo, slot, ro, t0o, t1o, k2, exo, h);
       pol.leaf(ok, h, o, work, off, mine);
       __syncwarp(mask);
-      if (mine > 0) {
+      if (kGroup || mine > 0) {
         nq = mine - min(mine, max(0, 32 - off));
         if (pol.enough()) {
           done = true;
           nq = 0;
         }
       }
+    } else if (kGroup) {
+      // ---- node step of groups: all lanes together
+      const int k0 = lane - gbase, m = tdone || done ? 0 : min(sp, gsize);
+      const bool act = k0 < m;
+      if (act) node = at(sp - 1 - k0);
+      sp -= m;
+      float tk[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+      int rk[4] = {-1, -1, -1, -1};
+      int nk = 0;
+      bool bad = act && unsigned(node) >= unsigned(sc.n_nodes);
+      if (act && !bad) {
+        float en[4];
+        int ch[4];
+        const unsigned hm = node4_test(sc.nodes4, node, ray, t0, t_far, en, ch);
+        ++ts.n_nodes;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (!((hm >> k) & 1u)) continue;
+          if (ch[k] < 0) {
+            if (unsigned(~ch[k]) >= unsigned(sc.n_prims)) {
+              bad = true;
+              continue;
+            }
+            ++ts.n_prims;
+            lq[nq * stride] = ~ch[k];  // nq <= kTrLeafQ - 4 here: a node adds at most four
+            ++nq;
+          } else {
+            tk[k] = en[k];
+            rk[k] = ch[k];
+            ++nk;
+          }
+        }
+        sort4(tk, rk);
+      }
+      // the children go on the stack, those of the group's first lane on top, the nearest of each last
+      const unsigned b0 = __ballot_sync(mask, (nk & 1) != 0) & glanes, b1 = __ballot_sync(mask, (nk & 2) != 0) & glanes,
+                     b2 = __ballot_sync(mask, (nk & 4) != 0) & glanes;
+      const unsigned above = lane == 31 ? 0u : ~0u << (lane + 1);
+      const int pushed = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+      const int base = sp + __popc(b0 & above) + 2 * __popc(b1 & above) + 4 * __popc(b2 & above);
+      const bool g_bad = (__ballot_sync(mask, bad) & glanes) != 0u;
+      const bool full = sp + pushed > (kTrStack - kTrLeafQ) << lg;
+      if (m > 0 && (g_bad || full)) {
+        ts.st = g_bad ? UGP_RAY_BAD_NODE : UGP_RAY_STACK_OVERFLOW;
+        tdone = true;
+        nq = 0;
+      } else if (m > 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (rk[k] >= 0) at(base + nk - 1 - k) = rk[k];  // hits are sorted first
+        sp += pushed;
+        if (sp == 0) tdone = true;
+      }
+      __syncwarp(mask);
     } else if (!done && !tdone) {
       if (unsigned(node) >= unsigned(sc.n_nodes)) {
         ts.st = UGP_RAY_BAD_NODE;
@@ -168,21 +237,27 @@ struct DepthSum {
   static constexpr bool kNearFirst = true;
   static constexpr float kScale = 1099511627776.f;  // 2^40
   static constexpr unsigned long long kOne = 1ull << 40;
-  unsigned long long* acc;
+  unsigned long long* acc;  // the warp's sums; a group's is its first lane's
+  int first;                // ~(lanes per ray - 1)
   __device__ void leaf(bool ok, const PrimHit& h, int o, bool, int, int) {
     if (ok)
-      atomicAdd(acc + (o - (int(threadIdx.x) & 31)),
+      atomicAdd(acc + (o & first),
                 (unsigned long long)__float2ll_rn(fminf(fmaxf(hit_half_integral(h), 0.f), 2.f) * kScale));
   }
-  __device__ bool enough() const { return *acc >= kOne; }  // saturated: T = 0 whatever follows
+  __device__ bool enough() const {  // saturated: T = 0 whatever follows
+    return *reinterpret_cast<volatile unsigned long long*>(acc + (int(threadIdx.x) & 31 & first)) >= kOne;
+  }
 };
+template <bool kGroup = false>
 static __device__ float tr_optical_depth(const TraceScene& sc, const Ray& ray, float t0, float t1, int ex,
                                          int* stk, int stride, unsigned long long* acc, int* owner, TrStats& ts,
-                                         bool live) {
-  DepthSum pol{acc};
+                                         bool live, int lg = 0) {
+  const int lane = int(threadIdx.x) & 31;
+  DepthSum pol{acc - lane, kGroup ? -(1 << lg) : -1};
   *acc = 0ull;
-  tr_walk(sc, ray, t0, t1, t1, ex, stk, stride, owner, ts, live, pol);
-  const unsigned long long a = *acc;
+  tr_walk<kGroup>(sc, ray, t0, t1, t1, ex, stk, stride, owner, ts, live, lg, pol);
+  __syncwarp();
+  const unsigned long long a = pol.acc[lane & pol.first];
   return a >= DepthSum::kOne ? 1.f : float(a) * (1.f / DepthSum::kScale);
 }
 
