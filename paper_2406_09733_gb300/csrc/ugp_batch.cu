@@ -231,12 +231,14 @@ struct BatchScanSrc {
   }
 };
 
+template <bool kFew>
 __global__ void __launch_bounds__(kFFBlock, kFFBlocksPerSM) k_b_extend(BState S) {
   __shared__ FFSmem sm;
   const BCtl& c = *S.ctl;
   const int cur = c.wave & 1;
   BatchScanSrc src{S, cur, c.live[cur], 0, 0, 0, 0, 0.f, 0.f, 0.f, TraceScene{}};
-  scan_persistent(sm, src, &S.ctl->scan_next);
+  if (kFew) scan_groups(sm, src, &S.ctl->scan_next, ff_group(src.count_));
+  else scan_persistent(sm, src, &S.ctl->scan_next);
 }
 
 __global__ void __launch_bounds__(128) k_b_shade(BState S) {
@@ -494,13 +496,13 @@ int grid_of(const void* kernel, int block, int64_t n) {
 // Persistent grid sizes of the wave kernels for a pool (computed before any stream capture).
 struct WaveGrids {
   int regen, ext, shade, shadow, retire;
-  bool few;  // shadow rays in groups of lanes
+  bool few, few_scan;  // shadow rays, free flights in groups of lanes
 };
 WaveGrids wave_grids(int64_t pool) {
-  const int ext_need = int((pool + kFFBlock / 32 - 1) / (kFFBlock / 32)), ext_cap = scan_grid((const void*)k_b_extend);
+  const int ext_need = int((pool + kFFBlock / 32 - 1) / (kFFBlock / 32)), ext_cap = scan_grid(pool <= kFFFew ? (const void*)k_b_extend<true> : (const void*)k_b_extend<false>);
   return WaveGrids{grid_of((const void*)k_b_regen, 256, pool), ext_need < ext_cap ? ext_need : ext_cap,
                    grid_of((const void*)k_b_shade, 128, pool), pool <= kTrFew ? tr_few_grid(pool) : tr_grid(pool),
-                   grid_of((const void*)k_b_retire, 256, pool), pool <= kTrFew};
+                   grid_of((const void*)k_b_retire, 256, pool), pool <= kTrFew, pool <= kFFFew};
 }
 
 // Launches one wave on `st` (also used while capturing the graph body).
@@ -508,7 +510,7 @@ ugp_status launch_wave(const BState& S, const WaveGrids& g, cudaGraphConditional
                        cudaStream_t st) {
   k_b_claim<<<1, 32, 0, st>>>(S);
   k_b_regen<<<g.regen, 256, 0, st>>>(S);
-  k_b_extend<<<g.ext, kFFBlock, 0, st>>>(S);
+  (g.few_scan ? k_b_extend<true> : k_b_extend<false>)<<<g.ext, kFFBlock, 0, st>>>(S);
   // every queued ray names its scene (S.dq.scenes), so the launch's own scene is unused
   ugp_status s = launch_dense(TraceScene{}, S.dq, 0, &S.ctl->dense_slots, S.pool, S.P.ps.prim, S.P.tu, S.P.ps.tsp,
                               nullptr, 0, nullptr, &S.ctl->dense_err, st);

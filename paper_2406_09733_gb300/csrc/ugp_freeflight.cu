@@ -44,7 +44,7 @@ struct ArrayScanSrc {
   }
 };
 
-template <bool STATS>
+template <bool STATS, bool kFew>
 __global__ void __launch_bounds__(kFFBlock, kFFBlocksPerSM)
 k_free_flight(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, const float* __restrict__ d3,
               const float* __restrict__ t0a, const float* __restrict__ t1a, const float* __restrict__ ua,
@@ -54,7 +54,8 @@ k_free_flight(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, const
   __shared__ FFSmem sm;
   ArrayScanSrc<STATS> src{sc, n_rays, o3, d3, t0a, t1a, ua, u2a, excl, prim_out, tu_out, tsp_out, st_out, ctr, dq,
                           0, 0.f, 0.f};
-  scan_persistent(sm, src, next);
+  if (kFew) scan_groups(sm, src, next, ff_group(n_rays));
+  else scan_persistent(sm, src, next);
 }
 
 }  // namespace
@@ -79,17 +80,13 @@ ugp_status launch_free_flight(const TraceScene& sc, int64_t n, const float* o3, 
     dq.list = reinterpret_cast<const int*>(static_cast<char*>(workspace) + dense_queue_bytes(n, slots));
   int* next = dq.count + 1;  // the scan's ray counter, in the queue header next to the queue length
   UGP_CUDA_CHECK(cudaMemsetAsync(dq.count, 0, 2 * sizeof(int), stream));
-  const void* kern = ctr ? (const void*)k_free_flight<true> : (const void*)k_free_flight<false>;
+  // the statistics count whole rays per lane
+  const auto kern = ctr ? k_free_flight<true, false> : (n <= kFFFew ? k_free_flight<false, true> : k_free_flight<false, false>);
   const int64_t need = (n + kFFBlock / 32 - 1) / (kFFBlock / 32);  // down to one ray per warp (rays_per_warp)
-  const int cap = scan_grid(kern);
+  const int cap = scan_grid((const void*)kern);
   const unsigned grid = unsigned(need < cap ? need : cap);
   prof_begin(kStQuery, stream);
-  if (ctr)
-    k_free_flight<true><<<grid, kFFBlock, 0, stream>>>(sc, n, o3, d3, t0, t1, u, u2, excl, prim, tu, tsp, st, ctr, dq,
-                                                      next);
-  else
-    k_free_flight<false><<<grid, kFFBlock, 0, stream>>>(sc, n, o3, d3, t0, t1, u, u2, excl, prim, tu, tsp, st, ctr, dq,
-                                                       next);
+  kern<<<grid, kFFBlock, 0, stream>>>(sc, n, o3, d3, t0, t1, u, u2, excl, prim, tu, tsp, st, ctr, dq, next);
   prof_end(kStQuery, stream);
   UGP_CUDA_CHECK(cudaGetLastError());
   return launch_dense(sc, dq, n, nullptr, n, prim, tu, tsp, st, 0, ctr, nullptr, stream);

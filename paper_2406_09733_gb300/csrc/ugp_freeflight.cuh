@@ -43,6 +43,8 @@
 // rays kept 10 of 32 lanes busy). A lane bins into the owning ray's bins with shared-memory atomics; the owner
 // moves its crossing bin after the step. Holding a primitive back can only delay a lowering of
 // the pruning limit, never skip a node that matters.
+#include <type_traits>
+
 #include "ugp_dense.cuh"
 #include "ugp_gauss.cuh"
 #include "ugp_philox.cuh"
@@ -187,6 +189,13 @@ struct OwnerRay {
 // primitives of the same ray in the same step); contributions to bins before the crossing bin
 // also go to the owner's running sum of them, and a primitive met before the crossing bin's end
 // goes into the owner's slot list. The owner moves its crossing bin afterwards.
+// With kGroup (up to 32 lanes bin for one ray at once) a bin or the running sum takes shares below
+// kBelowBig by plain additions, at most 32 at once on top of what the test before allows, and larger ones
+// one at a time (the bin) or as a request to sum the bins again (the running sum), so neither wraps.
+constexpr unsigned kBelowFull = 1u << 30, kBelowBig = 1u << 26;
+static_assert(kBelowFull + 32ull * kBelowBig < (1ull << 32) && 2ull * kBinCap + 32ull * kBelowBig < (1ull << 32),
+              "sums must not wrap");
+template <bool kGroup>
 static __device__ void pooled_leaf(FFSmem& sm, const OwnerRay& w, int slot, const PrimHit& h) {
   const float x = fmaxf(h.a, w.lo), y = fminf(h.b, w.hi);
   if (!(x < y)) return;
@@ -215,7 +224,12 @@ static __device__ void pooled_leaf(FFSmem& sm, const OwnerRay& w, int slot, cons
       const unsigned add = min(__float2uint_rn(fminf(fmaxf(amp * diff, 0.f) * kBinScale, 2.f * kBinScale)), kBinCap);
       unsigned* bp = &sm.bin[k][w.tid];
       if (add != 0u && *reinterpret_cast<volatile unsigned*>(bp) < kBinCap) {
-        atomicAdd(bp, add);
+        if (kGroup && add >= kBelowBig) {
+          unsigned old = *reinterpret_cast<volatile unsigned*>(bp), seen = ~old;
+          while (old < kBinCap && (seen = atomicCAS(bp, old, old + add)) != old) old = seen;
+        } else {
+          atomicAdd(bp, add);
+        }
         if (k < w.jc) dbelow += add;
       }
       tp = tq;
@@ -224,7 +238,15 @@ static __device__ void pooled_leaf(FFSmem& sm, const OwnerRay& w, int slot, cons
   }
   // a share above kBinCap makes the running sum exceed u anyway: capping it keeps the sum within
   // 32 bits
-  if (dbelow != 0ull) atomicAdd(&sm.below[w.tid], unsigned(dbelow < kBinCap ? dbelow : kBinCap));
+  if (dbelow != 0ull) {
+    if (!kGroup) {
+      atomicAdd(&sm.below[w.tid], unsigned(dbelow < kBinCap ? dbelow : kBinCap));
+    } else if (dbelow >= kBelowBig) {
+      atomicMax(&sm.below[w.tid], kBelowFull);
+    } else if (*reinterpret_cast<volatile unsigned*>(&sm.below[w.tid]) <= kBelowFull) {
+      atomicAdd(&sm.below[w.tid], unsigned(dbelow));
+    }
+  }
   if (x < w.edge(w.jc + 1) && w.list) {
     const int pos = atomicAdd(&sm.nlist[w.tid], 1);
     if (pos < kListCap) w.list[pos] = slot;
@@ -373,7 +395,8 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
       w.tid = (int(threadIdx.x) & ~31) | o;
       const int slot = work ? sm.lq[nq_o - 1 - (lane - off_o)][w.tid] : 0;
       PrimHit h;
-      if (prim_test_of<true>(work, w.prims, w.wlo, slot, w.ray, w.t0, w.t1, w.k2, w.ex, h)) pooled_leaf(sm, w, slot, h);
+      if (prim_test_of<true>(work, w.prims, w.wlo, slot, w.ray, w.t0, w.t1, w.k2, w.ex, h))
+        pooled_leaf<false>(sm, w, slot, h);
       __syncwarp();
       // each ray drops the items taken from the top of its queue and, when its running sum of
       // the bins before the crossing bin passes u, moves the crossing bin (bins are
@@ -453,6 +476,252 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
         --sp;
         node = sm.stk[sp][c.tid];
       }
+    }
+  }
+}
+
+// The scan for launches of few rays: 1 << lg neighbouring lanes share a ray, as in tr_walk (ugp_transmit.cuh).
+// The group's stack columns are one stack; a node step takes a node per lane from its top, and the
+// primitives met wait in each lane's own queue. The bins, sums and slot list are those of the group's first
+// lane, which also draws and writes the rays; the others hold copies of the ray, its bins' span and the
+// crossing bin. Taking several nodes at once is not quite nearest first, so a few more are visited before
+// the crossing is known; the result is the same function of (u, u2). Figures at ff_group.
+template <class Src>
+__device__ void scan_groups(FFSmem& sm, Src& src, int* next, int lg) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = int(threadIdx.x) & 31, wbase = int(threadIdx.x) & ~31, tid = int(threadIdx.x);
+  const int gsize = 1 << lg, gbase = lane & ~(gsize - 1), gtid = wbase | gbase;
+  const unsigned glanes = (gsize == 32 ? ~0u : (1u << gsize) - 1u) << gbase;
+  const unsigned below_me = (1u << lane) - 1u, above_me = lane == 31 ? 0u : ~0u << (lane + 1);
+  const bool head = lane == gbase;
+  auto at = [&](int i) -> int& { return sm.stk[i >> lg][gtid + (i & (gsize - 1))]; };
+  const int n = src.count();
+  const int groups = 32 >> lg;
+  const int used = min(groups, rays_per_warp(n, int64_t(gridDim.x) * (kFFBlock / 32)));
+  const int refill_at = max(1, used / 4);
+  ScanState s;
+  TraceScene sc = src.scene();
+  Ray ray = make_ray(make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 1.f));
+  float t0 = 0.f, t1 = 0.f, lo = 0.f, hi = 0.f, L = 0.f, target = 0.f, limit = 0.f;
+  int ex = -1, sp = 0, nq = 0, jc = kB;
+  unsigned n_nodes = 0u, n_prims = 0u;
+  uint8_t st = UGP_RAY_OK;
+  int* list = nullptr;
+  bool busy = false, exhausted = (lane >> lg) >= used, tdone = false;  // the same on all lanes of a group
+  for (;;) {
+    const unsigned waiting = __ballot_sync(kFull, busy && nq > 0);
+    const bool ready = busy && tdone && (waiting & glanes) == 0u;
+    const int mine = busy ? nq : 0;
+    const bool need_leaf = busy && (nq > kLeafQ - 4 || (tdone && nq > 0));
+    const unsigned sums = __reduce_add_sync(
+        kFull, unsigned(mine) | (busy && !ready ? 1u << 9 : 0u) |
+                   (head && (ready || (!busy && !exhausted)) ? 1u << 15 : 0u) | (need_leaf ? 1u << 21 : 0u));
+    const int total = int(sums & 511u), refill = int((sums >> 15) & 63u);
+    const bool urgent = (sums >> 21) != 0u;
+    bool working = ((sums >> 9) & 63u) != 0u;
+    if (refill >= refill_at || (refill > 0 && !working)) {
+      if (ready) {
+        if (head) {
+          s.lo = lo;
+          s.hi = hi;
+          s.jc = jc;
+          s.st = st;
+          s.n_nodes = n_nodes;
+          s.n_prims = n_prims;
+          s.nlist = sm.nlist[gtid];
+          src.finish(s, scan_result(sm, gtid, s, true));
+        }
+        busy = false;
+      }
+      __syncwarp();
+      const unsigned idle = __ballot_sync(kFull, head && !busy && !exhausted);
+      const int leader = __ffs(idle) - 1;
+      int base = 0;
+      if (lane == leader) base = atomicAdd(next, __popc(idle));
+      base = __shfl_sync(kFull, base, leader & 31);
+      int got = 0;  // 1: a ray to traverse, 2: no more rays
+      if (head && !busy && !exhausted) {
+        const int i = base + __popc(idle & below_me);
+        float u = 0.f;
+        if (i >= n) {
+          got = 2;
+        } else if (src.begin(i, s, u)) {
+          sc = src.scene();
+          lo = hi = s.t0;
+          if (sc.n_prims > 0 && s.t0 < s.t1) {
+            const float2 sp2 = scene_span(sc, s.ray, s.t0, s.t1);
+            lo = sp2.x;
+            hi = sp2.y;
+          }
+          if (!(lo < hi)) {  // nothing to traverse: the ray escapes
+            s.n_nodes = s.n_prims = 0u;
+            s.st = UGP_RAY_OK;
+            s.nlist = 0;
+            src.finish(s, scan_result(sm, gtid, s, false));
+          } else {
+            ray = s.ray;
+            t0 = s.t0;
+            t1 = s.t1;
+            ex = s.ex;
+            list = s.list;
+            target = u;
+            L = hi - lo;
+            got = 1;
+          }
+        }
+      }
+      got = __shfl_sync(kFull, got, gbase);
+      // the group's copies of what its first lane holds
+      auto f = [&](float& v) { v = __shfl_sync(kFull, v, gbase); };
+      f(ray.o.x); f(ray.o.y); f(ray.o.z); f(ray.d.x); f(ray.d.y); f(ray.d.z);
+      f(ray.inv.x); f(ray.inv.y); f(ray.inv.z); f(ray.inv_dd);
+      f(t0); f(t1); f(lo); f(hi); f(L);
+      ex = __shfl_sync(kFull, ex, gbase);
+      auto p = [&](auto*& v) {
+        v = reinterpret_cast<std::remove_reference_t<decltype(v)>>(
+            __shfl_sync(kFull, reinterpret_cast<unsigned long long>(v), gbase));
+      };
+      p(sc.nodes4); p(sc.prims); p(sc.wlo); p(list);
+      sc.n_prims = __shfl_sync(kFull, sc.n_prims, gbase);
+      sc.n_nodes = __shfl_sync(kFull, sc.n_nodes, gbase);
+      f(sc.k2);
+      if (got == 2) exhausted = true;
+      if (got == 1) {
+        for (int j = lane - gbase; j < kB; j += gsize) sm.bin[j][gtid] = 0u;
+        if (head) {
+          sm.below[gtid] = 0u;
+          sm.nlist[gtid] = 0;
+          at(0) = 0;
+        }
+        n_nodes = n_prims = 0u;
+        st = UGP_RAY_OK;
+        jc = kB;
+        limit = hi;
+        sp = 1;
+        nq = 0;
+        tdone = false;
+        busy = true;
+      }
+      __syncwarp();
+      working = __any_sync(kFull, busy);
+    }
+    if (!working) {
+      if (refill == 0) break;  // every group exhausted and its last ray written
+      continue;
+    }
+    if (total > 0 && (total >= 32 || urgent)) {
+      // ---- leaf step, as in scan_persistent
+      const unsigned q0 = __ballot_sync(kFull, (mine & 1) != 0), q1 = __ballot_sync(kFull, (mine & 2) != 0),
+                     q2 = __ballot_sync(kFull, (mine & 4) != 0), q3 = __ballot_sync(kFull, (mine & 8) != 0);
+      const int off = __popc(q0 & below_me) + 2 * __popc(q1 & below_me) + 4 * __popc(q2 & below_me) +
+                      8 * __popc(q3 & below_me);
+      const unsigned has = q0 | q1 | q2 | q3;
+      const unsigned starts = __reduce_or_sync(kFull, (mine > 0 && off < 32) ? (1u << off) : 0u);
+      const bool work = lane < total;
+      int* owner_of = sm.owner + wbase;
+      if (mine > 0) owner_of[__popc(has & below_me)] = lane;
+      __syncwarp();
+      const int o = work ? owner_of[__popc(starts & (0xffffffffu >> (31 - lane))) - 1] : lane;
+      const int off_o = __shfl_sync(kFull, off, o);
+      const int nq_o = __shfl_sync(kFull, mine, o);
+      OwnerRay w;
+      w.prims = reinterpret_cast<const float4*>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(sc.prims), o));
+      w.wlo = reinterpret_cast<const float4*>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(sc.wlo), o));
+      w.k2 = __shfl_sync(kFull, sc.k2, o);
+      w.ray.o = make_float3(__shfl_sync(kFull, ray.o.x, o), __shfl_sync(kFull, ray.o.y, o), __shfl_sync(kFull, ray.o.z, o));
+      w.ray.d = make_float3(__shfl_sync(kFull, ray.d.x, o), __shfl_sync(kFull, ray.d.y, o), __shfl_sync(kFull, ray.d.z, o));
+      w.ray.inv = make_float3(0.f, 0.f, 0.f);  // not used by the primitive test
+      w.ray.inv_dd = __shfl_sync(kFull, ray.inv_dd, o);
+      w.t0 = __shfl_sync(kFull, t0, o);
+      w.t1 = __shfl_sync(kFull, t1, o);
+      w.ex = __shfl_sync(kFull, ex, o);
+      w.lo = __shfl_sync(kFull, lo, o);
+      w.hi = __shfl_sync(kFull, hi, o);
+      w.L = __shfl_sync(kFull, L, o);
+      w.jc = __shfl_sync(kFull, jc, o);
+      w.list = reinterpret_cast<int*>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(list), o));
+      w.tid = wbase | (o & ~(gsize - 1));
+      const int slot = work ? sm.lq[nq_o - 1 - (lane - off_o)][wbase | o] : 0;
+      PrimHit h;
+      if (prim_test_of<true>(work, w.prims, w.wlo, slot, w.ray, w.t0, w.t1, w.k2, w.ex, h))
+        pooled_leaf<true>(sm, w, slot, h);
+      __syncwarp();
+      if (busy) nq = mine - min(mine, max(0, 32 - off));
+      // the crossing bin moves when the running sum passes u, or a large share asked for a look
+      const unsigned tgt = unsigned(target * kBinScale);
+      if (head && busy && sm.below[gtid] > tgt) {
+        unsigned long long acc = 0, before = 0;
+        int k = 0;
+        for (; k < jc; ++k) {
+          before = acc;
+          acc += sm.bin[k][gtid];
+          if (acc > tgt) break;
+        }
+        if (k < jc) {
+          jc = k;
+          acc = before;
+        }
+        sm.below[gtid] = unsigned(acc);  // exact again, at most u
+      }
+      __syncwarp();
+      const int jn = __shfl_sync(kFull, jc, gbase);
+      if (busy && (head || jn != jc)) {
+        jc = jn;
+        if (jc < kB) limit = bin_edge(lo, hi, L, jc + 1);
+      }
+    } else {
+      // ---- node step: a node per lane from the top of the group's stack, all lanes together
+      const int k0 = lane - gbase, m = busy && !tdone ? min(sp, gsize) : 0;
+      const bool act = k0 < m;
+      int node = 0;
+      if (act) node = at(sp - 1 - k0);
+      sp -= m;
+      float tk[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+      int rk[4] = {-1, -1, -1, -1};
+      int nk = 0;
+      bool bad = act && unsigned(node) >= unsigned(sc.n_nodes);
+      if (act && !bad) {
+        float en[4];
+        int ch[4];
+        const unsigned hm = node4_test(sc.nodes4, node, ray, lo, limit, en, ch);
+        ++n_nodes;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (!((hm >> k) & 1u)) continue;
+          if (ch[k] < 0) {
+            if (unsigned(~ch[k]) >= unsigned(sc.n_prims)) {
+              bad = true;
+              continue;
+            }
+            ++n_prims;
+            sm.lq[nq][tid] = ~ch[k];  // nq <= kLeafQ - 4 here: a node adds at most four
+            ++nq;
+          } else {
+            tk[k] = en[k];
+            rk[k] = ch[k];
+            ++nk;
+          }
+        }
+        sort4(tk, rk);
+      }
+      const unsigned b0 = __ballot_sync(kFull, (nk & 1) != 0) & glanes, b1 = __ballot_sync(kFull, (nk & 2) != 0) & glanes,
+                     b2 = __ballot_sync(kFull, (nk & 4) != 0) & glanes;
+      const int pushed = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+      const int base = sp + __popc(b0 & above_me) + 2 * __popc(b1 & above_me) + 4 * __popc(b2 & above_me);
+      const bool g_bad = (__ballot_sync(kFull, bad) & glanes) != 0u;
+      const bool full = sp + pushed > kFFStack << lg;
+      if (m > 0 && (g_bad || full)) {
+        st = g_bad ? UGP_RAY_BAD_NODE : UGP_RAY_STACK_OVERFLOW;
+        tdone = true;
+        nq = 0;
+      } else if (m > 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (rk[k] >= 0) at(base + nk - 1 - k) = rk[k];  // hits are sorted first; the nearest on top
+        sp += pushed;
+        if (sp == 0) tdone = true;
+      }
+      __syncwarp();
     }
   }
 }

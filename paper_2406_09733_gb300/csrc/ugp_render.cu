@@ -122,6 +122,7 @@ struct PathScanSrc {
   }
 };
 
+template <bool kFew>
 __global__ void __launch_bounds__(kFFBlock, kFFBlocksPerSM) k_extend(TraceScene sc, LightsDev L, uint2 key, int sample, int bounce,
                                                      int spawn_mode, PathSoA ps, const int* __restrict__ q,
                                                      const int* cnt, int* reset_next, int* reset_shadow, int* reset_shadow_e,
@@ -136,7 +137,8 @@ __global__ void __launch_bounds__(kFFBlock, kFFBlocksPerSM) k_extend(TraceScene 
     if (rays) atomicAdd(rays, (unsigned long long)count);
   }
   PathScanSrc src{sc, spawn_mode, count, ps, q, dq, rays, stats, 0, 0, 0, 0.f, 0.f, 0.f};
-  scan_persistent(sm, src, scan_next);
+  if (kFew) scan_groups(sm, src, scan_next, ff_group(count));
+  else scan_persistent(sm, src, scan_next);
 }
 
 template <bool kGuided>
@@ -643,7 +645,8 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
       UGP_CUDA_CHECK(cudaMemsetAsync(gs.L.c[9], 0, size_t(RL.E) * 4, st));
   }
   const int g_cam = grid_for((const void*)k_camera, 256, n);
-  const int g_ext = grid_for((const void*)k_extend, kFFBlock, 32 * n);  // down to one ray per warp
+  const auto extend = n <= kFFFew && !stats ? k_extend<true> : k_extend<false>;
+  const int g_ext = grid_for((const void*)extend, kFFBlock, 32 * n);  // down to one ray per warp
   const int g_shade = guide ? grid_for((const void*)k_shade<true>, 128, n) : grid_for((const void*)k_shade<false>, 128, n);
   // small images: groups of lanes per ray (the statistics count whole rays per lane)
   const bool few = n <= kTrFew && !stats;
@@ -659,7 +662,7 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
     for (int b = 0; b <= params->max_depth; ++b) {
       const int nxt = 1 - cur;
       prof_begin(kStExtend, st);
-      k_extend<<<g_ext, kFFBlock, 0, st>>>(sc, Ld, key, sample, b, params->spawn_mode, ps, queue[cur], counts + cur,
+      extend<<<g_ext, kFFBlock, 0, st>>>(sc, Ld, key, sample, b, params->spawn_mode, ps, queue[cur], counts + cur,
                                             counts + nxt, counts + 2, counts + 4, ray_counts, stats, dq, scan_next);
       prof_end(kStExtend, st);
       {

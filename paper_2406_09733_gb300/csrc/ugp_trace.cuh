@@ -58,6 +58,22 @@ inline int tr_few_grid(int64_t n) {
   return int((t + kTrBlock - 1) / kTrBlock);
 }
 
+// The same for the scan of free flights (kFFWarps resident warps on a GB300). Camera and bounce rays of a
+// 1M-primitive room, us for scan and finish, by lanes per ray:
+//   rays      1     4     8    16    32
+//     2K    454   231   179   159   149
+//     8K    624   351   296   266   262
+//    16K    805   479   396   378   397
+//    30K   1012   605   539   534   585
+//    60K   1152   816   798   853   973
+//   120K   1499  1272  1339  1477  1740
+//   250K   2266  2310  2532  2858  3428
+constexpr int kFFWarps = 152 * kFFBlocksPerSM * kFFBlock / 32;
+constexpr int kFFFew = 60 * kFFWarps;
+__host__ __device__ constexpr int ff_group(int64_t n) {
+  return n <= 3 * kFFWarps ? 5 : (n <= 10 * kFFWarps ? 4 : (n <= 25 * kFFWarps ? 3 : (n <= kFFFew ? 2 : 0)));
+}
+
 // Blocks of a transmittance launch of up to n rays.
 inline int tr_grid(int64_t n) {
   const int64_t full = (n + kTrBlock - 1) / kTrBlock;
