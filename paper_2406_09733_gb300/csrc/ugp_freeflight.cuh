@@ -670,8 +670,9 @@ __device__ void scan_groups(FFSmem& sm, Src& src, int* next, int lg) {
         if (jc < kB) limit = bin_edge(lo, hi, L, jc + 1);
       }
     } else {
-      // ---- node step: a node per lane from the top of the group's stack, all lanes together
-      const int k0 = lane - gbase, m = busy && !tdone ? min(sp, gsize) : 0;
+      // ---- node step: a node per lane from the top of the group's stack, all lanes together (one once
+      // the stack is half full: it then grows by three a level, as a single lane's does)
+      const int k0 = lane - gbase, m = busy && !tdone ? min(sp, sp > (kFFStack << lg) / 2 ? 1 : gsize) : 0;
       const bool act = k0 < m;
       int node = 0;
       if (act) node = at(sp - 1 - k0);

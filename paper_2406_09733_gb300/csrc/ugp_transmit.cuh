@@ -108,8 +108,9 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
         }
       }
     } else if (kGroup) {
-      // ---- node step of groups: all lanes together
-      const int k0 = lane - gbase, m = tdone || done ? 0 : min(sp, gsize);
+      // ---- node step of groups: all lanes together (one node once the stack is half full: it then
+      // grows by three a level, as a single lane's does)
+      const int k0 = lane - gbase, m = tdone || done ? 0 : min(sp, sp > ((kTrStack - kTrLeafQ) << lg) / 2 ? 1 : gsize);
       const bool act = k0 < m;
       if (act) node = at(sp - 1 - k0);
       sp -= m;
