@@ -185,13 +185,14 @@ __global__ void __launch_bounds__(256) k_b_regen(BState S) {
 // Rays of a wave: the live paths, each in its own request's scene. S refers to the kernel's
 // parameter (read through the constant bank, not copied into local memory).
 struct BatchScanSrc {
+  static constexpr bool kOneScene = false;
   const BState& S;
   int cur, count_;
   int i_, p, r, qf;
   float tq, u, u2;
   TraceScene sc;
   __device__ int count() const { return count_; }
-  __device__ TraceScene scene() const { return sc; }
+  __device__ const TraceScene& scene() const { return sc; }
   __device__ bool begin(int i, ScanState& s, float& uo) {
     i_ = i;
     p = S.live[cur][i];
@@ -356,7 +357,7 @@ __global__ void __launch_bounds__(kTrBlock, kTrBlocksPerSM) k_b_shadow(BState S)
     dist = S.sh.dist[j];
     ex = S.sh.excl[j];
   }
-  const float tau = tr_optical_depth<kFew>(sc, ray, 0.f, dist, ex, stk + threadIdx.x, kTrBlock, tr_acc + threadIdx.x,
+  const float tau = tr_optical_depth<kFew, false>(sc, ray, 0.f, dist, ex, stk + threadIdx.x, kTrBlock, tr_acc + threadIdx.x,
                                            tr_owner + threadIdx.x, ts, live, lg);
   if (!live || (lane & ((1 << lg) - 1)) != 0) return;
   const float T = fmaxf(0.f, 1.f - tau);

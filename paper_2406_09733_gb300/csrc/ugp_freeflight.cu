@@ -8,7 +8,8 @@ namespace {
 // Rays of a standalone query: caller arrays.
 template <bool STATS>
 struct ArrayScanSrc {
-  TraceScene sc;
+  static constexpr bool kOneScene = true;
+  const TraceScene& sc;
   int64_t n;
   const float *o3, *d3, *t0a, *t1a, *ua, *u2a;
   const int32_t* excl;
@@ -20,7 +21,7 @@ struct ArrayScanSrc {
   int cur;
   float u, u2;
   __device__ int count() const { return int(n); }
-  __device__ TraceScene scene() const { return sc; }
+  __device__ const TraceScene& scene() const { return sc; }
   __device__ bool begin(int i, ScanState& s, float& uo) {
     cur = i;
     s.ray = make_ray(ld3(o3, i), ld3(d3, i));

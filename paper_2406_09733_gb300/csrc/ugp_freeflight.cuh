@@ -155,12 +155,11 @@ static __device__ FFResult scan_result(FFSmem& sm, int tid, const ScanState& s, 
 // written as it ended), 7.38 at 4, 7.34 at 8, 7.37 at 12.
 constexpr int kRefill = 8;
 
-// Traversal context of one lane: the scene, the ray and its counters, as used by the
+// Traversal context of one lane: the ray and its counters, as used by the
 // persistent driver below.
 struct ScanCtx {
   FFSmem& sm;
   int tid;
-  TraceScene sc;
   Ray ray;
   float t0, t1;
   int ex;
@@ -257,7 +256,9 @@ static __device__ void pooled_leaf(FFSmem& sm, const OwnerRay& w, int slot, cons
 //   __device__ int count() const                    rays in this launch
 //   __device__ bool begin(int i, ScanState& s, float& u)   loads ray i (ray, t0, t1, ex, list);
 //                                                  false: the ray is skipped (no result)
-//   __device__ TraceScene scene() const             the current ray's scene
+//   __device__ const TraceScene& scene() const      the current ray's scene
+//   static constexpr bool kOneScene                 every ray has the same scene (a kernel parameter: its fields
+//                                                   are then read from the constant bank, not held or shuffled)
 //   __device__ void finish(const ScanState& s, const FFResult& r)   writes the current ray's result
 // Src is per thread and keeps what it needs of the current ray. `next` is a device counter,
 // zero before the launch. The node step is written out in the loop with the traversal state in
@@ -268,7 +269,7 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
   const int lane = int(threadIdx.x) & 31;
   constexpr unsigned kFull = 0xffffffffu;
   const int n = src.count();
-  ScanCtx c{sm, int(threadIdx.x), src.scene(), make_ray(make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 1.f)), 0.f,
+  ScanCtx c{sm, int(threadIdx.x), make_ray(make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 1.f)), 0.f,
             0.f, -1, 0u, 0u, UGP_RAY_OK, nullptr};
   ScanState s;
   const int used = rays_per_warp(n, int64_t(gridDim.x) * (kFFBlock / 32));
@@ -313,7 +314,6 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
         } else {
           float u = 0.f;
           if (src.begin(i, s, u)) {
-            c.sc = src.scene();
             c.ray = s.ray;
             c.t0 = s.t0;
             c.t1 = s.t1;
@@ -323,8 +323,8 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
             c.list = s.list;
             target = u;
             lo = hi = c.t0;
-            if (c.sc.n_prims > 0 && c.t0 < c.t1) {
-              const float2 sp2 = scene_span(c.sc, c.ray, c.t0, c.t1);
+            if (src.scene().n_prims > 0 && c.t0 < c.t1) {
+              const float2 sp2 = scene_span(src.scene(), c.ray, c.t0, c.t1);
               lo = sp2.x;
               hi = sp2.y;
             }
@@ -374,10 +374,17 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
       const int off_o = __shfl_sync(kFull, off, o);
       const int nq_o = __shfl_sync(kFull, mine, o);
       OwnerRay w;
-      w.prims = reinterpret_cast<const float4*>(
-          __shfl_sync(kFull, reinterpret_cast<unsigned long long>(c.sc.prims), o));
-      w.wlo = reinterpret_cast<const float4*>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(c.sc.wlo), o));
-      w.k2 = __shfl_sync(kFull, c.sc.k2, o);
+      if (Src::kOneScene) {
+        w.prims = src.scene().prims;
+        w.wlo = src.scene().wlo;
+        w.k2 = src.scene().k2;
+      } else {
+        w.prims = reinterpret_cast<const float4*>(
+            __shfl_sync(kFull, reinterpret_cast<unsigned long long>(src.scene().prims), o));
+        w.wlo = reinterpret_cast<const float4*>(
+            __shfl_sync(kFull, reinterpret_cast<unsigned long long>(src.scene().wlo), o));
+        w.k2 = __shfl_sync(kFull, src.scene().k2, o);
+      }
       w.ray.o = make_float3(__shfl_sync(kFull, c.ray.o.x, o), __shfl_sync(kFull, c.ray.o.y, o),
                             __shfl_sync(kFull, c.ray.o.z, o));
       w.ray.d = make_float3(__shfl_sync(kFull, c.ray.d.x, o), __shfl_sync(kFull, c.ray.d.y, o),
@@ -421,13 +428,13 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
       }
     } else if (busy && !tdone) {
       // ---- node step: one 4-wide node of the nearest-first traversal
-      if (unsigned(node) >= unsigned(c.sc.n_nodes)) {
+      if (unsigned(node) >= unsigned(src.scene().n_nodes)) {
         c.st = UGP_RAY_BAD_NODE;
         node = 0;
       }
       float en[4];
       int ch[4];
-      unsigned hm = node4_test(c.sc.nodes4, node, c.ray, lo, limit, en, ch);
+      unsigned hm = node4_test(src.scene().nodes4, node, c.ray, lo, limit, en, ch);
       ++c.n_nodes;
       float tk[4];
       int rk[4];
@@ -439,7 +446,7 @@ __device__ void scan_persistent(FFSmem& sm, Src& src, int* next) {
         if (!((hm >> k) & 1u)) continue;
         // a primitive's slot is checked here (its record is loaded by slot); a child node's
         // index is checked when it is visited
-        if (ch[k] < 0 && unsigned(~ch[k]) >= unsigned(c.sc.n_prims)) c.st = UGP_RAY_BAD_NODE;
+        if (ch[k] < 0 && unsigned(~ch[k]) >= unsigned(src.scene().n_prims)) c.st = UGP_RAY_BAD_NODE;
         if (c.st != UGP_RAY_OK) continue;
         if (ch[k] < 0) {
           ++c.n_prims;

@@ -99,7 +99,7 @@ k_radiance(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, const fl
     if (st_ff) st = __ldg(st_ff + r);
   }
   RadianceSum sum{em3, t_end, 0.f, 0.f, 0.f, 0.f};
-  tr_walk<false>(sc, ray, t0, t1, t_end, -1, stk + threadIdx.x, kTrBlock, owner + threadIdx.x, ts,
+  tr_walk<false, true>(sc, ray, t0, t1, t_end, -1, stk + threadIdx.x, kTrBlock, owner + threadIdx.x, ts,
                  live && st == UGP_RAY_OK, 0, sum);
   if (!live) return;
   const float rest = sat ? 0.f : fmaxf(0.f, 1.f - sum.mass);

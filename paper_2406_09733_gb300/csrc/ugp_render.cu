@@ -86,7 +86,8 @@ __global__ void __launch_bounds__(256) k_camera(CameraDev cam, LightsDev L, int 
 
 // Rays of a bounce: the live paths in the queue.
 struct PathScanSrc {
-  TraceScene sc;
+  static constexpr bool kOneScene = true;
+  const TraceScene& sc;
   int spawn_mode, count_;
   PathSoA ps;
   const int* q;
@@ -95,7 +96,7 @@ struct PathScanSrc {
   int i_, p, qf;
   float tq, u, u2;
   __device__ int count() const { return count_; }
-  __device__ TraceScene scene() const { return sc; }
+  __device__ const TraceScene& scene() const { return sc; }
   __device__ bool begin(int i, ScanState& s, float& uo) {
     i_ = i;
     p = q[i];

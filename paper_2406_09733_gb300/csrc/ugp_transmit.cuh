@@ -26,6 +26,8 @@ constexpr int kTrLeafQ = 10;  // primitives a lane may hold back (top of its sta
 // the ellipsoid's, and the shared recomputation of ill-conditioned hits took 1,000,003 light-sample rays
 // in a 1M-primitive room from 3.42 to 3.04 ms.
 //
+// With kOneScene all rays share the scene, whose fields then come from the constant bank.
+//
 // `P` collects the hits:
 //   leaf(bool ok, const PrimHit& h, int o, bool work, int off, int mine)   called by all lanes in a leaf
 //       step: this lane's primitive is hit (ok) by the ray of lane o; `work` lanes took a primitive, those
@@ -39,7 +41,7 @@ static_assert(kTrLeafQ < 16, "queue lengths are summed from four bit planes");
 // the group's first lane. A launch of few rays is bound by the chain of dependent steps of its longest
 // ray, and this shortens the chain, where spreading the rays over the warps left most lanes idle (figures at
 // tr_group).
-template <bool kGroup, class P>
+template <bool kGroup, bool kOneScene, class P>
 static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& ray, float t0, float t1, float t_far,
                                                int ex, int* stk, int stride, int* owner, TrStats& ts, bool live,
                                                int lg, P& pol) {
@@ -90,11 +92,13 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
       ro.inv_dd = __shfl_sync(mask, ray.inv_dd, o);
       const float t0o = __shfl_sync(mask, t0, o), t1o = __shfl_sync(mask, t1, o);
       const int exo = __shfl_sync(mask, ex, o);
-      const float4* prims = reinterpret_cast<const float4*>(
-          __shfl_sync(mask, reinterpret_cast<unsigned long long>(sc.prims), o));
-      const float4* wlo = reinterpret_cast<const float4*>(
-          __shfl_sync(mask, reinterpret_cast<unsigned long long>(sc.wlo), o));
-      const float k2 = __shfl_sync(mask, sc.k2, o);
+      const float4 *prims = sc.prims, *wlo = sc.wlo;
+      float k2 = sc.k2;
+      if (!kOneScene) {
+        prims = reinterpret_cast<const float4*>(__shfl_sync(mask, reinterpret_cast<unsigned long long>(prims), o));
+        wlo = reinterpret_cast<const float4*>(__shfl_sync(mask, reinterpret_cast<unsigned long long>(wlo), o));
+        k2 = __shfl_sync(mask, k2, o);
+      }
       PrimHit h;
       const int slot = work ? lq[(nq_o - 1 - (lane - off_o)) * stride + (o - lane)] : 0;
       const bool ok = prim_test_of<true>(work, prims, wlo, slot, ro, t0o, t1o, k2, exo, h);
@@ -249,14 +253,14 @@ struct DepthSum {
     return *reinterpret_cast<volatile unsigned long long*>(acc + (int(threadIdx.x) & 31 & first)) >= kOne;
   }
 };
-template <bool kGroup = false>
+template <bool kGroup = false, bool kOneScene = true>
 static __device__ float tr_optical_depth(const TraceScene& sc, const Ray& ray, float t0, float t1, int ex,
                                          int* stk, int stride, unsigned long long* acc, int* owner, TrStats& ts,
                                          bool live, int lg = 0) {
   const int lane = int(threadIdx.x) & 31;
   DepthSum pol{acc - lane, kGroup ? -(1 << lg) : -1};
   *acc = 0ull;
-  tr_walk<kGroup>(sc, ray, t0, t1, t1, ex, stk, stride, owner, ts, live, lg, pol);
+  tr_walk<kGroup, kOneScene>(sc, ray, t0, t1, t1, ex, stk, stride, owner, ts, live, lg, pol);
   __syncwarp();
   const unsigned long long a = pol.acc[lane & pol.first];
   return a >= DepthSum::kOne ? 1.f : float(a) * (1.f / DepthSum::kScale);
