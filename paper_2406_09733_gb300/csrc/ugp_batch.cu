@@ -233,12 +233,12 @@ struct BatchScanSrc {
 };
 
 template <bool kFew>
-__global__ void __launch_bounds__(kFFBlock, kFFBlocksPerSM) k_b_extend(BState S) {
-  __shared__ FFSmem sm;
+__global__ void __launch_bounds__(kFFBlock, kFFBlocksWide) k_b_extend(BState S) {
+  __shared__ FFSmem<kFFStack> sm;
   const BCtl& c = *S.ctl;
   const int cur = c.wave & 1;
   BatchScanSrc src{S, cur, c.live[cur], 0, 0, 0, 0, 0.f, 0.f, 0.f, TraceScene{}};
-  if (kFew) scan_groups(sm, src, &S.ctl->scan_next, ff_group(src.count_));
+  if constexpr (kFew) scan_groups(sm, src, &S.ctl->scan_next, ff_group(src.count_));
   else scan_persistent(sm, src, &S.ctl->scan_next);
 }
 

@@ -46,16 +46,16 @@ struct ArrayScanSrc {
 };
 
 template <bool STATS, bool kFew>
-__global__ void __launch_bounds__(kFFBlock, kFFBlocksPerSM)
+__global__ void __launch_bounds__(kFFBlock, kFew ? kFFBlocksWide : kFFBlocksPerSM)
 k_free_flight(TraceScene sc, int64_t n_rays, const float* __restrict__ o3, const float* __restrict__ d3,
               const float* __restrict__ t0a, const float* __restrict__ t1a, const float* __restrict__ ua,
               const float* __restrict__ u2a, const int32_t* __restrict__ excl,
               int32_t* __restrict__ prim_out, float* __restrict__ tu_out, float* __restrict__ tsp_out,
               uint8_t* __restrict__ st_out, unsigned long long* __restrict__ ctr, DenseQueue dq, int* next) {
-  __shared__ FFSmem sm;
+  __shared__ FFSmem<kFew ? kFFStack : kFFShort> sm;
   ArrayScanSrc<STATS> src{sc, n_rays, o3, d3, t0a, t1a, ua, u2a, excl, prim_out, tu_out, tsp_out, st_out, ctr, dq,
                           0, 0.f, 0.f};
-  if (kFew) scan_groups(sm, src, next, ff_group(n_rays));
+  if constexpr (kFew) scan_groups(sm, src, next, ff_group(n_rays));
   else scan_persistent(sm, src, next);
 }
 

@@ -124,12 +124,12 @@ struct PathScanSrc {
 };
 
 template <bool kFew>
-__global__ void __launch_bounds__(kFFBlock, kFFBlocksPerSM) k_extend(TraceScene sc, LightsDev L, uint2 key, int sample, int bounce,
+__global__ void __launch_bounds__(kFFBlock, kFew ? kFFBlocksWide : kFFBlocksPerSM) k_extend(TraceScene sc, LightsDev L, uint2 key, int sample, int bounce,
                                                      int spawn_mode, PathSoA ps, const int* __restrict__ q,
                                                      const int* cnt, int* reset_next, int* reset_shadow, int* reset_shadow_e,
                                                      unsigned long long* rays, unsigned long long* stats,
                                                      DenseQueue dq, int* scan_next) {
-  __shared__ FFSmem sm;
+  __shared__ FFSmem<kFew ? kFFStack : kFFShort> sm;
   const int count = load_count(cnt);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *reset_next = 0;
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kFFBlock, kFFBlocksPerSM) k_extend(TraceScene 
     if (rays) atomicAdd(rays, (unsigned long long)count);
   }
   PathScanSrc src{sc, spawn_mode, count, ps, q, dq, rays, stats, 0, 0, 0, 0.f, 0.f, 0.f};
-  if (kFew) scan_groups(sm, src, scan_next, ff_group(count));
+  if constexpr (kFew) scan_groups(sm, src, scan_next, ff_group(count));
   else scan_persistent(sm, src, scan_next);
 }
 

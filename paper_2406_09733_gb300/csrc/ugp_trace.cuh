@@ -10,7 +10,9 @@ constexpr int kTrStack = 48;       // transmittance: traversal stack depth
 constexpr int kTrBlocksPerSM = 8;  // transmittance: resident blocks per SM (24 KB shared, <= 64 registers)
 constexpr int kFFBlock = 128;      // free flight: threads per block of the scan
 constexpr int kFFStack = 36;       // free flight: traversal stack depth (4-wide nodes)
-constexpr int kFFBlocksPerSM = 5;  // free flight: resident scan blocks per SM (41 KB shared, <= 102 registers)
+constexpr int kFFShort = 26;       // of it in shared memory where six blocks of the scan share an SM
+constexpr int kFFBlocksPerSM = 6;  // free flight: resident scan blocks per SM (37 KB shared, <= 80 registers)
+constexpr int kFFBlocksWide = 5;   // the same for scans with more state (groups, a scene per ray; 42 KB, <= 102)
 constexpr int kB = 32;             // free flight: bins of the scan
 constexpr int kTrWarps = 152 * kTrBlocksPerSM * kTrBlock / 32;  // warps of the transmittance a GB300 holds
 
@@ -68,7 +70,7 @@ inline int tr_few_grid(int64_t n) {
 //    60K   1152   816   798   853   973
 //   120K   1499  1272  1339  1477  1740
 //   250K   2266  2310  2532  2858  3428
-constexpr int kFFWarps = 152 * kFFBlocksPerSM * kFFBlock / 32;
+constexpr int kFFWarps = 152 * kFFBlocksWide * kFFBlock / 32;
 constexpr int kFFFew = 60 * kFFWarps;
 __host__ __device__ constexpr int ff_group(int64_t n) {
   return n <= 3 * kFFWarps ? 5 : (n <= 10 * kFFWarps ? 4 : (n <= 25 * kFFWarps ? 3 : (n <= kFFFew ? 2 : 0)));
