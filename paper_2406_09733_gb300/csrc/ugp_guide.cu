@@ -47,37 +47,37 @@ __global__ void __launch_bounds__(256) k_guide_pack(const float* __restrict__ pa
   }
 }
 
-// Sums the blocks' partials in a fixed order: thread (p, k) of a block adds those of blocks k, k + 8, ... of
-// parameter p, then eight of these are added. One thread per parameter left 76 blocks of 152 serial loads
-// each, 11 us for 152 partials; this takes 5.
+// Sums the blocks' partials in block order (Adam divides by the gradient's own size, so the rounding of a
+// nearly cancelling sum is kept as it is): eight threads per parameter bring its partials into shared memory,
+// one adds them. One thread per parameter, loading and adding, left 76 blocks of 152 serial loads each, 11 us
+// for 152 partials; this takes 5.
 constexpr int kRedParams = 32, kRedParts = 8;
 __global__ void __launch_bounds__(kRedParams * kRedParts) k_guide_reduce(const float* __restrict__ partial, int grid,
                                                                          float* __restrict__ grad,
                                                                          const float* __restrict__ loss_partial,
                                                                          float* __restrict__ loss) {
-  __shared__ float sum[kRedParts][kRedParams];
+  __shared__ float v[kGMaxGradBlocks][kRedParams];
+  __shared__ float lv[kGMaxGradBlocks];
   const int x = int(threadIdx.x) % kRedParams, k = int(threadIdx.x) / kRedParams;
   const int p = int(blockIdx.x) * kRedParams + x;
-  float s = 0.f;
-  if (p < UGP_GUIDE_NPARAMS) {
-#pragma unroll 4
-    for (int c = k; c < grid; c += kRedParts) s += partial[size_t(c) * UGP_GUIDE_NPARAMS + p];
-  }
-  sum[k][x] = s;
+  const bool with_loss = loss && blockIdx.x == 0;
+#pragma unroll 8
+  for (int c = k; c < grid; c += kRedParts) v[c][x] = p < UGP_GUIDE_NPARAMS ? partial[size_t(c) * UGP_GUIDE_NPARAMS + p] : 0.f;
+  if (with_loss && int(threadIdx.x) < grid) lv[threadIdx.x] = loss_partial[threadIdx.x];
   __syncthreads();
   if (k == 0 && p < UGP_GUIDE_NPARAMS) {
-#pragma unroll
-    for (int j = 1; j < kRedParts; ++j) s += sum[j][x];
+    float s = 0.f;
+#pragma unroll 8
+    for (int c = 0; c < grid; ++c) s += v[c][x];
     grad[p] = s;
   }
-  if (loss && blockIdx.x == 0 && k == 1) {  // one warp: lane x adds every 32nd, then a tree
-    float t = 0.f;
-    for (int c = x; c < grid; c += kRedParams) t += loss_partial[c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (x == 0) *loss = t;
+  if (with_loss && threadIdx.x == kRedParams) {  // another warp's
+    float s = 0.f;
+    for (int c = 0; c < grid; ++c) s += lv[c];
+    *loss = s;
   }
 }
+static_assert(kGMaxGradBlocks <= kRedParams * kRedParts, "a thread per loss partial");
 
 __global__ void __launch_bounds__(256) k_guide_adam(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
                                                     const float* __restrict__ g, float lr, float b1, float b2, float eps,
