@@ -53,50 +53,55 @@ struct GuideCfgDev {
 
 __device__ __forceinline__ float clamp01(float v) { return fminf(1.f, fmaxf(0.f, v)); }
 
-// The 64 input features of a vertex.
-__device__ __forceinline__ void guide_encode(const GuideCfgDev& c, float3 x, float3 wo, float f[kGWidth]) {
-  const float xn[3] = {clamp01((x.x - c.lo.x) * c.inv_ext.x), clamp01((x.y - c.lo.y) * c.inv_ext.y),
-                       clamp01((x.z - c.lo.z) * c.inv_ext.z)};
+// Features of one coordinate: sin/cos(2^l angle) for l < kN, with the pair for l = 0 given. The higher
+// frequencies by double angles: sin 2a = 2 sin a cos a, cos 2a = (cos a - sin a)(cos a + sin a); five
+// doublings leave an error of a few 1e-6, far below the BF16 step the layer input is rounded to.
+template <int kN>
+__device__ __forceinline__ void double_angles(float s, float co, float* f) {
+#pragma unroll
+  for (int l = 0; l < kN; ++l) {
+    f[2 * l] = s;
+    f[2 * l + 1] = co;
+    const float s2 = 2.f * s * co;
+    co = (co - s) * (co + s);
+    s = s2;
+  }
+}
+__device__ __forceinline__ float3 guide_position(const GuideCfgDev& c, float3 x) {
+  return f3(clamp01((x.x - c.lo.x) * c.inv_ext.x), clamp01((x.y - c.lo.y) * c.inv_ext.y),
+            clamp01((x.z - c.lo.z) * c.inv_ext.z));
+}
+// Features 12 a .. 12 a + 11 of position coordinate a (in [0, 1]).
+__device__ __forceinline__ void encode_axis(float xn, float* f) {
+  float s, co;
+  sincospif(xn, &s, &co);
+  double_angles<6>(s, co, f);
+}
+// Features 36 .. 63: the angles of wo, the raw values, zeros.
+__device__ __forceinline__ void encode_rest(float3 xn, float3 wo, float* f) {
   const float theta = acosf(fminf(1.f, fmaxf(-1.f, wo.z)));
   const float phi = atan2f(wo.y, wo.x);
-  // the higher frequencies by double angles: sin 2a = 2 sin a cos a, cos 2a = (cos a - sin a)
-  // (cos a + sin a); five doublings leave an error of a few 1e-6, far below the BF16 step the
-  // layer input is rounded to
-  int i = 0;
+  float s, co;
+  sincosf(theta, &s, &co);
+  double_angles<4>(s, co, f);
+  sincosf(phi, &s, &co);
+  double_angles<4>(s, co, f + 8);
+  f[16] = xn.x;
+  f[17] = xn.y;
+  f[18] = xn.z;
+  f[19] = theta * 0.318309886183790672f;         // theta / pi
+  f[20] = phi * 0.159154943091895336f + 0.5f;    // phi / (2 pi) + 1/2
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    float s, co;
-    sincospif(xn[a], &s, &co);
-#pragma unroll
-    for (int l = 0; l < 6; ++l) {
-      f[i++] = s;
-      f[i++] = co;
-      const float s2 = 2.f * s * co;
-      co = (co - s) * (co + s);
-      s = s2;
-    }
-  }
-  const float ang[2] = {theta, phi};
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    float s, co;
-    sincosf(ang[a], &s, &co);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      f[i++] = s;
-      f[i++] = co;
-      const float s2 = 2.f * s * co;
-      co = (co - s) * (co + s);
-      s = s2;
-    }
-  }
-  f[i++] = xn[0];
-  f[i++] = xn[1];
-  f[i++] = xn[2];
-  f[i++] = theta * 0.318309886183790672f;         // theta / pi
-  f[i++] = phi * 0.159154943091895336f + 0.5f;    // phi / (2 pi) + 1/2
-#pragma unroll
-  for (; i < kGWidth;) f[i++] = 0.f;
+  for (int i = 21; i < 28; ++i) f[i] = 0.f;
+}
+
+// The 64 input features of a vertex.
+__device__ __forceinline__ void guide_encode(const GuideCfgDev& c, float3 x, float3 wo, float f[kGWidth]) {
+  const float3 xn = guide_position(c, x);
+  encode_axis(xn.x, f);
+  encode_axis(xn.y, f + 12);
+  encode_axis(xn.z, f + 24);
+  encode_rest(xn, wo, f + 36);
 }
 
 __device__ __forceinline__ float softplusf(float s) { return fmaxf(s, 0.f) + log1pf(expf(-fabsf(s))); }
@@ -166,54 +171,60 @@ __device__ __forceinline__ float3 mixture_sample(const float mix[kGOut], float u
   return normalize3((1.f - omw) * mu + (s * cp) * t + (s * sp) * b);
 }
 
-// Loss -w ln q(wi) of one sample and its gradient with respect to the 40 head outputs.
-__device__ __forceinline__ float mixture_loss_grad(const GuideCfgDev& c, const float Y[kGOut], float3 wi, float w,
-                                                   float dY[kGOut]) {
-  float amax = -3.4e38f;
+// The loss -w ln q(wi) of one sample and its gradient with respect to the head outputs, by kLoss lobes per
+// thread, kGLobes / kLoss threads per sample. Y: the 5 kLoss head outputs of this thread's lobes; A: the
+// weights' outputs of all lobes. Stage 1 gives each lobe's log of pi_j v_j(wi); with all of them in
+// ell[0 .. kGLobes), stage 2 gives the gradient (over Y) and returns the loss.
+template <int kLoss>
+struct LobeLoss {
+  float cw[kLoss], in[kLoss], k[kLoss];
+  bool free_k[kLoss];
+  float logz;
+  __device__ void stage1(const GuideCfgDev& c, const float* Y, const float A[kGLobes], float3 wi, float* ell) {
+    float amax = -3.4e38f;
 #pragma unroll
-  for (int j = 0; j < kGLobes; ++j) amax = fmaxf(amax, Y[5 * j + 4]);
-  float z = 0.f;
+    for (int j = 0; j < kGLobes; ++j) amax = fmaxf(amax, A[j]);
+    float z = 0.f;
 #pragma unroll
-  for (int j = 0; j < kGLobes; ++j) z += expf(Y[5 * j + 4] - amax);
-  const float logz = amax + logf(z);
-  float ell[kGLobes];
-  float lmax = -3.4e38f;
+    for (int j = 0; j < kGLobes; ++j) z += expf(A[j] - amax);
+    logz = amax + logf(z);
 #pragma unroll
-  for (int j = 0; j < kGLobes; ++j) {
-    const float mx = Y[5 * j], my = Y[5 * j + 1], mz = Y[5 * j + 2];
-    const float n = sqrtf(mx * mx + my * my + mz * mz);
-    const float in = n > 0.f ? 1.f / n : 0.f;
-    const float cw = n > 0.f ? (mx * wi.x + my * wi.y + mz * wi.z) * in : wi.z;
-    const float kr = c.kappa_min + softplusf(Y[5 * j + 3]);
-    const float k = fminf(kr, c.kappa_max);
-    ell[j] = (Y[5 * j + 4] - logz) + vmf_log_norm(k) + k * (cw - 1.f);
-    lmax = fmaxf(lmax, ell[j]);
-    // stash what the second pass needs in dY
-    dY[5 * j] = cw;
-    dY[5 * j + 1] = in;
-    dY[5 * j + 2] = k;
-    dY[5 * j + 3] = kr > c.kappa_max ? 0.f : 1.f;
+    for (int j = 0; j < kLoss; ++j) {
+      const float mx = Y[5 * j], my = Y[5 * j + 1], mz = Y[5 * j + 2];
+      const float n = sqrtf(mx * mx + my * my + mz * mz);
+      in[j] = n > 0.f ? 1.f / n : 0.f;
+      cw[j] = n > 0.f ? (mx * wi.x + my * wi.y + mz * wi.z) * in[j] : wi.z;
+      const float kr = c.kappa_min + softplusf(Y[5 * j + 3]);
+      k[j] = fminf(kr, c.kappa_max);
+      free_k[j] = !(kr > c.kappa_max);
+      ell[j] = (Y[5 * j + 4] - logz) + vmf_log_norm(k[j]) + k[j] * (cw[j] - 1.f);
+    }
   }
-  float sq = 0.f;
+  // own: this thread's entries of ell
+  __device__ float stage2(float* Y, const float ell[kGLobes], const float* own, float3 wi, float w) {
+    float lmax = -3.4e38f;
 #pragma unroll
-  for (int j = 0; j < kGLobes; ++j) sq += expf(ell[j] - lmax);
-  const float logq = lmax + logf(sq);
+    for (int j = 0; j < kGLobes; ++j) lmax = fmaxf(lmax, ell[j]);
+    float sq = 0.f;
 #pragma unroll
-  for (int j = 0; j < kGLobes; ++j) {
-    const float cw = dY[5 * j], in = dY[5 * j + 1], k = dY[5 * j + 2], free_k = dY[5 * j + 3];
-    const float r = expf(ell[j] - logq);
-    const float pi = expf(Y[5 * j + 4] - logz);
-    dY[5 * j + 4] = w * (pi - r);
-    const float dlk = 1.f / k - 2.f / expm1f(2.f * k) + (cw - 1.f);
-    const float sig = 1.f / (1.f + expf(-Y[5 * j + 3]));
-    dY[5 * j + 3] = free_k * (-w * r * dlk * sig);
-    const float g = -w * r * k * in;
-    const float mx = Y[5 * j] * in, my = Y[5 * j + 1] * in, mz = Y[5 * j + 2] * in;
-    dY[5 * j] = g * (wi.x - cw * mx);
-    dY[5 * j + 1] = g * (wi.y - cw * my);
-    dY[5 * j + 2] = g * (wi.z - cw * mz);
+    for (int j = 0; j < kGLobes; ++j) sq += expf(ell[j] - lmax);
+    const float logq = lmax + logf(sq);
+#pragma unroll
+    for (int j = 0; j < kLoss; ++j) {
+      const float r = expf(own[j] - logq);
+      const float pi = expf(Y[5 * j + 4] - logz);
+      Y[5 * j + 4] = w * (pi - r);
+      const float dlk = 1.f / k[j] - 2.f / expm1f(2.f * k[j]) + (cw[j] - 1.f);
+      const float sig = 1.f / (1.f + expf(-Y[5 * j + 3]));
+      Y[5 * j + 3] = free_k[j] ? -w * r * dlk * sig : 0.f;
+      const float g = -w * r * k[j] * in[j];
+      const float mx = Y[5 * j] * in[j], my = Y[5 * j + 1] * in[j], mz = Y[5 * j + 2] * in[j];
+      Y[5 * j] = g * (wi.x - cw[j] * mx);
+      Y[5 * j + 1] = g * (wi.y - cw[j] * my);
+      Y[5 * j + 2] = g * (wi.z - cw[j] * mz);
+    }
+    return -w * logq;
   }
-  return -w * logq;
-}
+};
 
 }  // namespace ugp

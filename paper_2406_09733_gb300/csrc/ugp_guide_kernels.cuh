@@ -1,9 +1,9 @@
 // Tensor-core kernels of the learned guide (tcgen05.mma with TMEM accumulators, operands in
 // shared memory, weights brought in by one bulk TMA copy per block).
 //
-// A block of 128 threads owns tiles of 128 rows (vertices); thread t owns row t, which is
-// tensor-memory lane t of the M = 128 accumulator, so every epilogue is a per-thread
-// tcgen05.ld of its own row. Per layer one thread issues four K = 16 MMAs
+// A tile is 128 rows (vertices); row t is tensor-memory lane t of the M = 128 accumulator, and
+// every epilogue is a tcgen05.ld by the threads that own the row (one in the forward kernel, four
+// in training). Per layer one thread issues four K = 16 MMAs
 // (D[128 x 64] = X[128 x 64] W^T), commits them to an mbarrier, and all threads wait with a
 // time limit (a wait that gives up sets the workspace's error word and the block leaves
 // through its single exit, which frees its tensor memory).
@@ -92,17 +92,24 @@ __device__ __forceinline__ void store_row(uint8_t* tile, int r, const float (&v)
   }
 }
 
-// Reads row r of a 128-row BF16 tile as raw 16-bit values.
-__device__ __forceinline__ void load_row_bits(const uint8_t* tile, int r, uint16_t (&h)[kGWidth]) {
+// 0xffff in each half of a BF16 pair that is above zero.
+__device__ __forceinline__ uint32_t positive_mask(uint32_t pair) {
+  return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&pair), __floats2bfloat162_rn(0.f, 0.f));
+}
+// Writes columns c, c + 1 (c even) of row r of a 128-row tile as BF16.
+__device__ __forceinline__ void store_pair(uint8_t* tile, int r, int c, float a, float b) {
+  *reinterpret_cast<uint32_t*>(tile + tile_off(uint32_t(r), uint32_t(c), 128u)) = pack_bf16x2(a, b);
+}
+// Writes columns c .. c + 15 (c a multiple of 8) of row r of a 128-row tile as BF16.
+__device__ __forceinline__ void store_part(uint8_t* tile, int r, int c, const float (&v)[16]) {
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const uint4 q = *reinterpret_cast<const uint4*>(tile + tile_off(uint32_t(r), uint32_t(8 * c), 128u));
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      h[8 * c + 2 * j] = uint16_t(w[j] & 0xffffu);
-      h[8 * c + 2 * j + 1] = uint16_t(w[j] >> 16);
-    }
+  for (int k = 0; k < 2; ++k) {
+    uint4 q;
+    q.x = pack_bf16x2(v[8 * k], v[8 * k + 1]);
+    q.y = pack_bf16x2(v[8 * k + 2], v[8 * k + 3]);
+    q.z = pack_bf16x2(v[8 * k + 4], v[8 * k + 5]);
+    q.w = pack_bf16x2(v[8 * k + 6], v[8 * k + 7]);
+    *reinterpret_cast<uint4*>(tile + tile_off(uint32_t(r), uint32_t(c + 8 * k), 128u)) = q;
   }
 }
 
@@ -135,12 +142,15 @@ __device__ __forceinline__ Operand mnmajor(const uint8_t* tile, uint32_t R) {
   return {smem_u32(tile), 128u, R * 16u, 256u};
 }
 
-// Issues D = A B^T (+ D) over `ksteps` K = 16 slices. Called by one thread.
-__device__ __forceinline__ void issue(uint32_t d, const Operand& a, const Operand& b, int ksteps, uint32_t idesc,
-                                      bool accumulate) {
-  for (int ks = 0; ks < ksteps; ++ks)
-    mma_bf16(d, desc_smem(a.addr + uint32_t(ks) * a.kstep, a.lbo, a.sbo),
-             desc_smem(b.addr + uint32_t(ks) * b.kstep, b.lbo, b.sbo), idesc, (accumulate || ks > 0) ? 1u : 0u);
+// Issues D = A B^T (+ D) over kSteps K = 16 slices. Called by one thread. A slice's descriptor is the first's
+// with its address field (in units of 16 bytes) advanced.
+template <int kSteps>
+__device__ __forceinline__ void issue(uint32_t d, const Operand& a, const Operand& b, uint32_t idesc, bool accumulate) {
+  const uint64_t da = desc_smem(a.addr, a.lbo, a.sbo), db = desc_smem(b.addr, b.lbo, b.sbo);
+#pragma unroll
+  for (int ks = 0; ks < kSteps; ++ks)
+    mma_bf16(d, da + uint64_t(ks) * (a.kstep >> 4), db + uint64_t(ks) * (b.kstep >> 4), idesc,
+             (accumulate || ks > 0) ? 1u : 0u);
 }
 
 __device__ __forceinline__ int64_t row_count(int64_t n_host, const int* n_dev) {
@@ -256,7 +266,7 @@ __global__ void __launch_bounds__(kGThreads * kFwdGroups, 1) k_guide_fwd(GuideDe
       group_sync(grp);
       if (t == 0) {
         tc_fence_after();
-        issue(tmem, kmajor(X, 128), kmajor(sm + kImgW + l * kImgTile, 64), 4, kIdescFwd, false);
+        issue<4>(tmem, kmajor(X, 128), kmajor(sm + kImgW + l * kImgTile, 64), kIdescFwd, false);
         mma_commit(gbar);
       }
       const bool ok = mbar_wait(gbar, phase, kGWaitNs);
@@ -337,7 +347,8 @@ constexpr uint32_t kGrX = kGrDZ + kXTile;               // 58624: X_0 .. X_4
 constexpr uint32_t kGrBar = kGrX + 5 * kGrXTile;        // 161024
 constexpr uint32_t kGrTmemSlot = kGrBar + 8;
 constexpr uint32_t kGrRed = kGrBar + 16;                // 4 floats of loss reduction
-constexpr uint32_t kGrSmem = kGrBar + 128;              // 161152
+constexpr uint32_t kGrEx = kGrBar + 128;                // per row: 8 weight outputs, 8 log terms of the lobes
+constexpr uint32_t kGrSmem = kGrEx + 2 * kGLobes * 128 * 4;
 static_assert(kGrSmem <= 227 * 1024, "guide training block exceeds shared memory");
 // The dW MMA's M = 128 view of dZ reads 16 column chunks, the upper 8 (unused accumulator lanes)
 // up to 16 KB past the dZ tile; that range is X_0, inside the block's shared memory.
@@ -347,18 +358,27 @@ constexpr uint32_t kTmScratch = 0;   // 64 columns: layer output / dX
 constexpr uint32_t kTmDW = 64;       // 5 x 80 columns: dW_l and db_l
 constexpr uint32_t kTmCols = 512;
 
+// A row's work between the products (encoding, bias and ReLU, the loss gradient, the masked dZ) is shared
+// by kParts threads, each with its 16 of 64 columns, its 2 of 8 lobes and its piece of the encoding; the
+// lobes' terms that all of them need go through shared memory. With a thread per row (4 warps per SM, ten
+// dependent products and 5,700 instructions per tile) 65,536 rows took 61 us, with four
+// 52; an optimiser step of 1,000,000 rows 621 us, now 476.
+constexpr int kParts = 4;
+constexpr int kGrThreads = kGThreads * kParts;
+static_assert(kGLobes % kParts == 0 && kGWidth == 16 * kParts, "columns and lobes per thread");
+
 // Src: __device__ bool sample(int64_t row, float3& x, float3& wo, float3& wi, float& w) const
 template <class Src>
-__global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src, int64_t n_host, const int* n_dev,
+__global__ void __launch_bounds__(kGrThreads, 1) k_guide_grad(GuideDev g, Src src, int64_t n_host, const int* n_dev,
                                                              float* __restrict__ partial,
                                                              float* __restrict__ loss_partial) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  const int tid = int(threadIdx.x), warp = tid >> 5;
+  const int tid = int(threadIdx.x), warp = tid >> 5, t = tid & (kGThreads - 1), part = tid / kGThreads;
   const int64_t n = row_count(n_host, n_dev);
   const int64_t ntiles = (n + kGThreads - 1) / kGThreads;
   float* my_partial = partial + size_t(blockIdx.x) * UGP_GUIDE_NPARAMS;
   if (int64_t(blockIdx.x) >= ntiles) {
-    for (int p = tid; p < UGP_GUIDE_NPARAMS; p += kGThreads) my_partial[p] = 0.f;
+    for (int p = tid; p < UGP_GUIDE_NPARAMS; p += kGrThreads) my_partial[p] = 0.f;
     if (tid == 0) loss_partial[blockIdx.x] = 0.f;
     return;
   }
@@ -368,6 +388,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src
   const uint32_t bar = smem_u32(sm + kGrBar);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kGrTmemSlot);
   float* red = reinterpret_cast<float*>(sm + kGrRed);
+  float* ex = reinterpret_cast<float*>(sm + kGrEx);
   if (tid == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
@@ -379,17 +400,17 @@ __global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src
   // Columns 64..79 of every X_l: a ones column (bias gradient) and zeros; written once.
   {
     const uint4 ones = make_uint4(pack_bf16x2(1.f, 0.f), 0u, 0u, 0u), zeros = make_uint4(0u, 0u, 0u, 0u);
-    for (int l = 0; l <= kGLayers; ++l) {
-      uint8_t* t = X + l * kGrXTile;
-      *reinterpret_cast<uint4*>(t + tile_off(uint32_t(tid), 64u, 128u)) = ones;
-      *reinterpret_cast<uint4*>(t + tile_off(uint32_t(tid), 72u, 128u)) = zeros;
+    for (int l = part; l <= kGLayers; l += kParts) {
+      uint8_t* xt = X + l * kGrXTile;
+      *reinterpret_cast<uint4*>(xt + tile_off(uint32_t(t), 64u, 128u)) = ones;
+      *reinterpret_cast<uint4*>(xt + tile_off(uint32_t(t), 72u, 128u)) = zeros;
     }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  const uint32_t lane_addr = tmem + (uint32_t(warp * 32) << 16);
+  const uint32_t lane_addr = tmem + (uint32_t((warp & 3) * 32) << 16);
   uint32_t phase = 0;
   if (tid == 0) {
     mbar_expect_tx(bar, kImgBytes);
@@ -401,19 +422,23 @@ __global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src
   float loss_acc = 0.f;
   bool first = true;
   for (int64_t tile = blockIdx.x; tile < ntiles && !failed; tile += gridDim.x) {
-    const int64_t row = tile * kGThreads + tid;
+    const int64_t row = tile * kGThreads + t;
     float3 x = f3(0.f, 0.f, 0.f), wo = f3(0.f, 0.f, 1.f), wi = f3(0.f, 0.f, 1.f);
     float w = 0.f;
     const bool valid = row < n && src.sample(row, x, wo, wi, w);
     {
-      float f[kGWidth];
-      if (valid) {
-        guide_encode(g.cfg, x, wo, f);
-      } else {
+      const float3 xn = guide_position(g.cfg, x);
+      if (part < 3) {
+        float f[12];
+        if (valid) encode_axis(part == 0 ? xn.x : (part == 1 ? xn.y : xn.z), f);
 #pragma unroll
-        for (int i = 0; i < kGWidth; ++i) f[i] = 0.f;
+        for (int i = 0; i < 12; i += 2) store_pair(X, t, 12 * part + i, valid ? f[i] : 0.f, valid ? f[i + 1] : 0.f);
+      } else {
+        float f[28];
+        if (valid) encode_rest(xn, wo, f);
+#pragma unroll
+        for (int i = 0; i < 28; i += 2) store_pair(X, t, 36 + i, valid ? f[i] : 0.f, valid ? f[i + 1] : 0.f);
       }
-      store_row(X, tid, f);
     }
     // forward
     for (int l = 0; l <= kGLayers && !failed; ++l) {
@@ -422,8 +447,8 @@ __global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src
       __syncthreads();
       if (tid == 0) {
         tc_fence_after();
-        issue(tmem + kTmScratch, kmajor(X + l * kGrXTile, 128), kmajor(sm + kImgW + l * kImgTile, 64), 4, kIdescFwd,
-              false);
+        issue<4>(tmem + kTmScratch, kmajor(X + l * kGrXTile, 128), kmajor(sm + kImgW + l * kImgTile, 64), kIdescFwd,
+                 false);
         mma_commit(bar);
       }
       const bool ok = mbar_wait(bar, phase, kGWaitNs);
@@ -434,27 +459,43 @@ __global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src
       }
       tc_fence_after();
       if (l < kGLayers) {
-        float v[kGWidth];
-        tmem_row<kGWidth>(lane_addr + kTmScratch, v);
+        float v[16];
+        tmem_row<16>(lane_addr + kTmScratch + 16u * uint32_t(part), v);
 #pragma unroll
-        for (int i = 0; i < kGWidth; ++i) v[i] = fmaxf(v[i] + bias[l * kGWidth + i], 0.f);
-        store_row(X + (l + 1) * kGrXTile, tid, v);
+        for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i] + bias[l * kGWidth + 16 * part + i], 0.f);
+        store_part(X + (l + 1) * kGrXTile, t, 16 * part, v);
       } else {
-        float v[48];
-        tmem_row<48>(lane_addr + kTmScratch, v);
-        float Y[kGOut], dY[kGOut];
+        constexpr int kLoss = kGLobes / kParts, kY = 5 * kLoss;
+        float v[16], Y[kY];
+        tmem_row<16>(lane_addr + kTmScratch + uint32_t(kY * part), v);
 #pragma unroll
-        for (int i = 0; i < kGOut; ++i) Y[i] = v[i] + bias[kGLayers * kGWidth + i];
-        if (valid && w != 0.f) {
-          loss_acc += mixture_loss_grad(g.cfg, Y, wi, w * inv_n, dY);
-        } else {
+        for (int i = 0; i < kY; ++i) Y[i] = v[i] + bias[kGLayers * kGWidth + kY * part + i];
+        float *ex_a = ex + t, *ex_l = ex + kGLobes * 128 + t;  // columns of 128 rows
 #pragma unroll
-          for (int i = 0; i < kGOut; ++i) dY[i] = 0.f;
+        for (int j = 0; j < kLoss; ++j) ex_a[(kLoss * part + j) * 128] = Y[5 * j + 4];
+        __syncthreads();
+        const bool use = valid && w != 0.f;
+        float A[kGLobes], own[kLoss];
+        LobeLoss<kLoss> loss;
+#pragma unroll
+        for (int j = 0; j < kGLobes; ++j) A[j] = ex_a[j * 128];
+        if (use) {
+          loss.stage1(g.cfg, Y, A, wi, own);
+#pragma unroll
+          for (int j = 0; j < kLoss; ++j) ex_l[(kLoss * part + j) * 128] = own[j];
         }
-        float d64[kGWidth];
+        __syncthreads();
+        if (use) {
 #pragma unroll
-        for (int i = 0; i < kGWidth; ++i) d64[i] = i < kGOut ? dY[i] : 0.f;
-        store_row(DZ, tid, d64);
+          for (int j = 0; j < kGLobes; ++j) A[j] = ex_l[j * 128];
+          const float lv = loss.stage2(Y, A, own, wi, w * inv_n);
+          if (part == 0) loss_acc += lv;
+        }
+#pragma unroll
+        for (int i = 0; i < kY; i += 2) store_pair(DZ, t, kY * part + i, use ? Y[i] : 0.f, use ? Y[i + 1] : 0.f);
+        constexpr int kPad = (kGWidth - kGOut) / kParts;  // columns past the head, zero
+#pragma unroll
+        for (int i = 0; i < kPad; i += 2) store_pair(DZ, t, kGOut + kPad * part + i, 0.f, 0.f);
       }
     }
     // backward, head first
@@ -464,10 +505,9 @@ __global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src
       __syncthreads();
       if (tid == 0) {
         tc_fence_after();
-        issue(tmem + kTmDW + 80u * uint32_t(l), mnmajor(DZ, 128), mnmajor(X + l * kGrXTile, 128), 8, kIdescDW,
-              !first);
+        issue<8>(tmem + kTmDW + 80u * uint32_t(l), mnmajor(DZ, 128), mnmajor(X + l * kGrXTile, 128), kIdescDW, !first);
         if (l > 0)
-          issue(tmem + kTmScratch, kmajor(DZ, 128), mnmajor(sm + kImgW + l * kImgTile, 64), 4, kIdescDX, false);
+          issue<4>(tmem + kTmScratch, kmajor(DZ, 128), mnmajor(sm + kImgW + l * kImgTile, 64), kIdescDX, false);
         mma_commit(bar);
       }
       const bool ok = mbar_wait(bar, phase, kGWaitNs);
@@ -478,32 +518,40 @@ __global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src
       }
       if (l > 0) {
         tc_fence_after();
-        float v[kGWidth];
-        tmem_row<kGWidth>(lane_addr + kTmScratch, v);
-        uint16_t h[kGWidth];
-        load_row_bits(X + l * kGrXTile, tid, h);  // X_l = relu(Z_{l-1}) rounded: > 0 iff Z_{l-1} > 0
+        float v[16];
+        tmem_row<16>(lane_addr + kTmScratch + 16u * uint32_t(part), v);
+        // X_l = relu(Z_{l-1}) rounded: > 0 iff Z_{l-1} > 0; masked as packed pairs
 #pragma unroll
-        for (int i = 0; i < kGWidth; ++i) v[i] = (h[i] != 0 && !(h[i] & 0x8000u)) ? v[i] : 0.f;
-        store_row(DZ, tid, v);
+        for (int c = 0; c < 2; ++c) {
+          const uint32_t off = tile_off(uint32_t(t), uint32_t(16 * part + 8 * c), 128u);
+          const uint4 q = *reinterpret_cast<const uint4*>(X + l * kGrXTile + off);
+          uint4 z;
+          z.x = pack_bf16x2(v[8 * c], v[8 * c + 1]) & positive_mask(q.x);
+          z.y = pack_bf16x2(v[8 * c + 2], v[8 * c + 3]) & positive_mask(q.y);
+          z.z = pack_bf16x2(v[8 * c + 4], v[8 * c + 5]) & positive_mask(q.z);
+          z.w = pack_bf16x2(v[8 * c + 6], v[8 * c + 7]) & positive_mask(q.w);
+          *reinterpret_cast<uint4*>(DZ + off) = z;
+        }
       }
     }
     first = false;
   }
-  // Block partials: lanes 0..63 of the dW accumulators (warps 0 and 1) hold the output rows.
+  // Block partials: lanes 0..63 of the dW accumulators (warps 0 and 1 of each part) hold the output rows;
+  // a thread writes 16 of its row's 64 columns, part 0 the bias column as well.
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (!failed && warp < 2) {
-    const int o = tid;
+  if (!failed && t < 64) {
 #pragma unroll 1
     for (int l = 0; l <= kGLayers; ++l) {
-      float v[80];
-      tmem_row<80>(lane_addr + kTmDW + 80u * uint32_t(l), v);
-      if (o < guide_out_dim(l)) {
-        float* pw = my_partial + guide_w_off(l) + o * kGWidth;
+      float v[16], vb[16];
+      tmem_row<16>(lane_addr + kTmDW + 80u * uint32_t(l) + 16u * uint32_t(part), v);
+      tmem_row<16>(lane_addr + kTmDW + 80u * uint32_t(l) + 64u, vb);
+      if (t < guide_out_dim(l)) {
+        float* pw = my_partial + guide_w_off(l) + t * kGWidth + 16 * part;
 #pragma unroll
-        for (int i = 0; i < kGWidth; ++i) pw[i] = first ? 0.f : v[i];
-        my_partial[guide_b_off(l) + o] = first ? 0.f : v[64];
+        for (int i = 0; i < 16; ++i) pw[i] = first ? 0.f : v[i];
+        if (part == 0) my_partial[guide_b_off(l) + t] = first ? 0.f : vb[0];
       }
     }
   }
@@ -512,7 +560,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_guide_grad(GuideDev g, Src src
     float s = loss_acc;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if ((tid & 31) == 0) red[warp] = s;
+    if ((tid & 31) == 0 && part == 0) red[warp] = s;
     __syncthreads();
     if (tid == 0) loss_partial[blockIdx.x] = failed ? 0.f : red[0] + red[1] + red[2] + red[3];
   }
@@ -562,7 +610,7 @@ ugp_status launch_guide_grad(const GuideDev& g, const Src& src, int64_t n_host, 
   int64_t cap = guide_sm_count();
   if (cap > kGMaxGradBlocks - 1) cap = kGMaxGradBlocks - 1;
   const int grid = int(tiles < cap ? (tiles > 0 ? tiles : 1) : cap);
-  kern<<<grid, kGThreads, gk::kGrSmem, st>>>(g, src, n_host, n_dev, ws.partial, ws.loss_partial);
+  kern<<<grid, gk::kGrThreads, gk::kGrSmem, st>>>(g, src, n_host, n_dev, ws.partial, ws.loss_partial);
   UGP_CUDA_CHECK(cudaGetLastError());
   *grid_out = grid;
   return UGP_OK;
