@@ -121,7 +121,7 @@ __global__ void k_b_init(BState S, int n_req, unsigned long long items_total, in
     c.rays = rays;
     c.dense_err = 0ull;
     c.scan_next = 0;
-    *S.dq.count = 0;
+    S.dq.count[2] = 0;
     c.start_ns = umma::global_timer_ns();
   }
 }
@@ -405,7 +405,7 @@ __global__ void k_b_cond(BState S, cudaGraphConditionalHandle handle, int use_gr
   c.shadow = 0;
   c.retire = 0;
   c.scan_next = 0;
-  *S.dq.count = 0;
+  S.dq.count[2] = 0;
   c.wave += 1;
   int more = (c.live[nxt] > 0 || c.work_next < c.items_total) ? 1 : 0;
   if (more && c.wave >= c.max_waves) {

@@ -619,7 +619,6 @@ ugp_status launch_dense(const TraceScene& sc, const DenseQueue& q, int64_t n_hos
   if (ps != UGP_OK) return ps;
   auto cap_grid = [](int64_t need, int cap) { return unsigned(need < cap ? (need > 0 ? need : 1) : cap); };
   const Outputs O{prim_out, t_u_out, t_spawn_out, status_out, spawn_mode, stats, rays_err};
-  UGP_CUDA_CHECK(cudaMemsetAsync(q.count + 2, 0, 2 * sizeof(int), stream));
   prof_begin(kStDense, stream);
   k_dense<<<cap_grid((max_slots + 2 * kDWarps - 1) / (2 * kDWarps), g_dense_grid), 32 * kDWarps,
             sizeof(WarpSmem) * kDWarps, stream>>>(sc, q, n_host, n_dev, O);

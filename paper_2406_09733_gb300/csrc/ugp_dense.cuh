@@ -12,8 +12,8 @@ namespace ugp {
 
 // Structure of arrays in caller-provided scratch memory (a 256-byte header, then the columns).
 struct DenseQueue {
-  int* count;    // header ints: [0] unused, [1] ray counter of the persistent scan, [2] and [3]
-                 // rays handed to the finish's second and third passes
+  int* count;    // header ints: [0] unused, [1] ray counter of the persistent scan, [2] rays handed to the
+                 // finish's second pass (zero before launch_dense), [3] unused
   int* idx;      // output index of the ray (-1: empty slot)
   float *lo, *hi, *Flo, *u, *u2;
   float *ox, *oy, *oz, *dx, *dy, *dz, *t0, *t1;
@@ -98,6 +98,7 @@ __device__ __forceinline__ void dense_none(const DenseQueue& q, int j) { q.idx[j
 ugp_status dense_prepare();
 // Slots 0 .. n-1 are walked, n = *n_dev when n_dev is not NULL, else n_host; max_slots bounds n
 // (grid size).
+// q.count[2] must be zero: a caller clears it with its other counters, in a kernel that runs in between anyway.
 ugp_status launch_dense(const TraceScene& sc, const DenseQueue& q, int64_t n_host, const int* n_dev,
                         int64_t max_slots, int* prim_out, float* t_u_out, float* t_spawn_out, uint8_t* status_out,
                         int spawn_mode, unsigned long long* stats, unsigned long long* rays_err, cudaStream_t stream);

@@ -80,7 +80,7 @@ ugp_status launch_free_flight(const TraceScene& sc, int64_t n, const float* o3, 
   if (with_lists)
     dq.list = reinterpret_cast<const int*>(static_cast<char*>(workspace) + dense_queue_bytes(n, slots));
   int* next = dq.count + 1;  // the scan's ray counter, in the queue header next to the queue length
-  UGP_CUDA_CHECK(cudaMemsetAsync(dq.count, 0, 2 * sizeof(int), stream));
+  UGP_CUDA_CHECK(cudaMemsetAsync(dq.count, 0, 4 * sizeof(int), stream));
   // the statistics count whole rays per lane
   const auto kern = ctr ? k_free_flight<true, false> : (n <= kFFFew ? k_free_flight<false, true> : k_free_flight<false, false>);
   const int64_t need = (n + kFFBlock / 32 - 1) / (kFFBlock / 32);  // down to one ray per warp (rays_per_warp)

@@ -657,7 +657,7 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
   for (int si = 0; si < params->spp; ++si) {
     const int sample = params->spp_begin + si;
     prof_begin(kStCamera, st);
-    k_camera<<<g_cam, 256, 0, st>>>(cd, Ld, int(n), key, sample, ps, queue[0], counts + 0, dq.count, scan_next);
+    k_camera<<<g_cam, 256, 0, st>>>(cd, Ld, int(n), key, sample, ps, queue[0], counts + 0, dq.count + 2, scan_next);
     prof_end(kStCamera, st);
     int cur = 0;
     for (int b = 0; b <= params->max_depth; ++b) {
@@ -682,12 +682,12 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
       prof_begin(kStShade, st);
       if (guide)
         k_shade<true><<<g_shade, 128, 0, st>>>(md, Ld, key, sample, b, params->max_depth, params->nee, ps, queue[cur],
-                                                counts + cur, queue[nxt], counts + nxt, sh, counts + 2, she, counts + 4, dq.count,
+                                                counts + cur, queue[nxt], counts + nxt, sh, counts + 2, she, counts + 4, dq.count + 2,
                                                 scan_next, gs, Em);
       else
         k_shade<false><<<g_shade, 128, 0, st>>>(md, Ld, key, sample, b, params->max_depth, params->nee, ps,
                                                  queue[cur], counts + cur, queue[nxt], counts + nxt, sh, counts + 2, she, counts + 4,
-                                                 dq.count, scan_next, gs, Em);
+                                                 dq.count + 2, scan_next, gs, Em);
       prof_end(kStShade, st);
       // one launch per kind of light sample: a path's two shadow rays add to its radiance in
       // this order, so the sum does not depend on scheduling
