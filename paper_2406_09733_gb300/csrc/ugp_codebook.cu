@@ -63,10 +63,14 @@ __global__ void k_init_book(int64_t n, const float* __restrict__ X, float* __res
 
 // Fixed-point sums and counts of the points of every entry of group G. Points share few entries (a wall has
 // one normal and one size, a cluster one material), so atomics to global memory queue on them: 2.0 ms for
-// the SGGX of 1M points, 1.4 for their materials. A block sums its points in shared memory first, kAccDims
+// the SGGX of 1M points, 1.4 for their materials. A block sums its points in shared memory first, acc_dims
 // values at a time (blockIdx.y), once per warp where all its points have the same entry, and adds what it
-// found to global memory.
-constexpr int kAccThreads = 512;
+// found to global memory. An addition of 64 bits in shared memory is a loop that tries until no other
+// lane came between, so the sums are kept as two words of 32 bits: the low kAccBits of the values, which
+// 2^15 of them cannot carry out of a word, and the rest (materials of 1M points: 0.48 -> 0.10 ms).
+// Values from 512 up, whose rest could overflow, go to global memory as they are.
+constexpr int kAccThreads = 512, kAccLog = 15, kAccBits = 32 - kAccLog;
+constexpr int kAccRounds = (1 << kAccLog) / kAccThreads;  // 2^15 points per block between write-outs
 template <int G>
 constexpr int acc_dims() { return kDim[G] <= 4 ? kDim[G] : (kDim[G] == 6 ? 3 : 4); }
 template <int G>
@@ -77,40 +81,56 @@ __global__ void __launch_bounds__(kAccThreads, 1) k_accumulate(int64_t n, const 
                                                                unsigned long long* __restrict__ sums,
                                                                unsigned int* __restrict__ cnt) {
   constexpr int D = kDim[G], O = kOff[G], N = acc_dims<G>();
-  extern __shared__ unsigned long long acc[];  // N x kCodes, then the counts
-  unsigned* num = reinterpret_cast<unsigned*>(acc + N * kCodes);
+  extern __shared__ unsigned acc[];  // of N x kCodes sums the low words, then the high ones; then the counts
+  unsigned* high = acc + N * kCodes;
+  unsigned* num = high + N * kCodes;
   const int lane = threadIdx.x & 31, d0 = int(blockIdx.y) * N;
-  for (int k = threadIdx.x; k < kCodes; k += kAccThreads) {
-    for (int d = 0; d < N; ++d) acc[d * kCodes + k] = 0ull;
-    num[k] = 0u;
-  }
-  __syncthreads();
-  for (int64_t i0 = int64_t(blockIdx.x) * kAccThreads; i0 < n; i0 += int64_t(gridDim.x) * kAccThreads) {
-    const int64_t i = i0 + threadIdx.x;
-    const int k = i < n ? int(code[i]) : -1;
-    long long v[N];
+  const int64_t step = int64_t(gridDim.x) * kAccThreads;
+  for (int64_t i1 = int64_t(blockIdx.x) * kAccThreads; i1 < n; i1 += step * kAccRounds) {
+    for (int k = threadIdx.x; k < kCodes; k += kAccThreads) {
+      for (int d = 0; d < N; ++d) acc[d * kCodes + k] = high[d * kCodes + k] = 0u;
+      num[k] = 0u;
+    }
+    __syncthreads();
+    const int64_t end = n < i1 + step * kAccRounds ? n : i1 + step * kAccRounds;
+    for (int64_t i0 = i1; i0 < end; i0 += step) {
+      const int64_t i = i0 + threadIdx.x;
+      const int k = i < n ? int(code[i]) : -1;
+      long long v[N];
 #pragma unroll
-    for (int d = 0; d < N; ++d) v[d] = k >= 0 ? __float2ll_rn(X[i * kFeat + O + d0 + d] * kFix) : 0ll;
-    const int k0 = __shfl_sync(0xffffffffu, k, 0);
-    if (__all_sync(0xffffffffu, k == k0)) {
-      if (k0 < 0) continue;
+      for (int d = 0; d < N; ++d) v[d] = k >= 0 ? __float2ll_rn(X[i * kFeat + O + d0 + d] * kFix) : 0ll;
+      const int k0 = __shfl_sync(0xffffffffu, k, 0);
+      const bool one = __all_sync(0xffffffffu, k == k0);
+      if (one) {
+#pragma unroll
+        for (int d = 0; d < N; ++d)
+          for (int o = 16; o > 0; o >>= 1) v[d] += __shfl_xor_sync(0xffffffffu, v[d], o);
+      }
+      if (k < 0) continue;
 #pragma unroll
       for (int d = 0; d < N; ++d) {
-        for (int o = 16; o > 0; o >>= 1) v[d] += __shfl_xor_sync(0xffffffffu, v[d], o);
-        if (lane == d) atomicAdd(acc + d * kCodes + k0, (unsigned long long)v[d]);
+        if (one && lane != d) continue;
+        const long long h = v[d] >> kAccBits;
+        if (h < -(1 << (31 - kAccLog)) || h >= 1 << (31 - kAccLog)) {
+          atomicAdd(sums + size_t(k) * D + d0 + d, (unsigned long long)v[d]);
+        } else {
+          atomicAdd(acc + d * kCodes + k, unsigned(v[d]) & ((1u << kAccBits) - 1u));
+          atomicAdd(high + d * kCodes + k, unsigned(int(h)));
+        }
       }
-      if (lane == 0) atomicAdd(num + k0, 32u);
-    } else if (k >= 0) {
-#pragma unroll
-      for (int d = 0; d < N; ++d) atomicAdd(acc + d * kCodes + k, (unsigned long long)v[d]);
-      atomicAdd(num + k, 1u);
+      if (!one) atomicAdd(num + k, 1u);
+      else if (lane == 0) atomicAdd(num + k, 32u);
     }
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < kCodes; k += kAccThreads) {
-    if (num[k] == 0u) continue;
-    for (int d = 0; d < N; ++d) atomicAdd(sums + size_t(k) * D + d0 + d, acc[d * kCodes + k]);
-    if (blockIdx.y == 0) atomicAdd(cnt + k, num[k]);
+    __syncthreads();
+    for (int k = threadIdx.x; k < kCodes; k += kAccThreads) {
+      if (num[k] == 0u) continue;
+      for (int d = 0; d < N; ++d) {
+        const long long v = ((long long)int(high[d * kCodes + k]) << kAccBits) + acc[d * kCodes + k];
+        atomicAdd(sums + size_t(k) * D + d0 + d, (unsigned long long)v);
+      }
+      if (blockIdx.y == 0) atomicAdd(cnt + k, num[k]);
+    }
+    __syncthreads();
   }
 }
 

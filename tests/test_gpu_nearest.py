@@ -74,3 +74,34 @@ def test_codes_are_those_of_the_scan(ugp, n, kind):
     for g, (o, w) in GROUPS.items():
         ref = _scan(torch, X[g], book[:, o:o + w].contiguous()).cpu().numpy()
         assert np.array_equal(got[g], ref), (g, np.flatnonzero(got[g] != ref)[:5])
+
+
+@pytest.mark.parametrize("n", [1, 4097, 1_400_000])
+def test_entries_are_the_means_of_their_points(ugp, n):
+    """Sums of values that fit the words of shared memory, at their limit (512) and beyond, over more points
+    than one pass holds: the fixed-point sums are whole numbers, so the entries are equal."""
+    import torch
+    rng = np.random.Generator(np.random.Philox(n))
+    row = rng.normal(size=(300, 22)).astype(np.float32)
+    row[:, 10:13] = rng.choice(np.array([-600, -511.99, 0, 300, 511.99, 512, 1e5], np.float32), (300, 3))
+    row[:, 0] *= np.where(rng.random(300) < 0.1, np.float32(700), np.float32(1))
+    pick = np.where(np.arange(n) < n // 2, np.arange(n) * 100 // max(n, 1), rng.integers(0, 300, n))
+    x = row[pick]                                       # runs of equal points, then points in any order
+    s = scenes.room_scene(100, seed=1, n_clusters=3).subset(np.arange(100)[:1])
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+    rep = lambda a: t(np.repeat(a, n, 0))
+    mats = ugp.Materials(t(x[:, :6]), torch.zeros(n, dtype=torch.uint8).cuda(), t(x[:, 6:9]), t(x[:, 9]),
+                         t(x[:, 10:13]), t(x[:, 13:22]))
+    book, _ = ugp.codebook_encode(rep(s.mean), rep(s.quat), rep(s.scale), rep(s.magnitude), mats, iters=1)
+    got = book.cpu().numpy()
+    first = x[np.arange(4096, dtype=np.int64) * n // 4096]
+    for o, w, c in ((7, 6, 0), (13, 16, 6)):
+        code = _scan(torch, t(row[:, c:c + w]), t(first[:, c:c + w])).cpu().numpy()[pick]
+        num = np.bincount(code, minlength=4096)
+        want = first[:, c:c + w].copy()
+        for d in range(w):
+            v = np.rint(x[:, c + d] * np.float32(2 ** 24)).astype(np.int64)
+            total = np.zeros(4096, np.int64)
+            np.add.at(total, code, v)
+            want[num > 0, d] = (total[num > 0].astype(np.float64) / (2.0 ** 24 * num[num > 0])).astype(np.float32)
+        assert np.array_equal(got[:, o:o + w], want), o
