@@ -236,9 +236,9 @@ ugp_status fit_group(int64_t n, const float* X, float* book, uint16_t* code, cha
   UGP_CUDA_CHECK(cudaFuncSetAttribute(nearest::k_assign<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmem)));
   char* p = ws + L.book;
   nearest::Scratch S;
-  S.tbook = reinterpret_cast<float*>(p);
-  S.packed = reinterpret_cast<uint8_t*>(p + size_t(16) * kCodes * 4);
-  S.perm = reinterpret_cast<int*>(p + size_t(16) * kCodes * 4 + size_t(kCodes) * 64 * 2);
+  S.tbook = reinterpret_cast<float4*>(p);
+  S.packed = reinterpret_cast<uint8_t*>(p + size_t(5) * kCodes * 16);
+  S.perm = reinterpret_cast<int*>(p + size_t(5) * kCodes * 16 + size_t(kCodes) * 64 * 2);
   S.center = reinterpret_cast<float*>(reinterpret_cast<char*>(S.perm) + size_t(kCodes) * 4);
   S.cmax = reinterpret_cast<unsigned*>(ws + L.cmax);
   S.dead = reinterpret_cast<uint8_t*>(ws + L.dead);
