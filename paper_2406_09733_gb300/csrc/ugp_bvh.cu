@@ -6,11 +6,10 @@
 //                      the k-ellipsoid, block-reduced centroid bounds
 //   2. k_morton        30-bit Morton code of each box centre
 //   3. radix sort      (ugp_sort.cu, on the caller's workspace) of (code, index), stable
-//   4. k_hierarchy     binary radix tree over the sorted codes (Karras, HPG 2012)
+//   4. k_tree          binary radix tree over the sorted codes and its boxes, from the leaves up
 //   5. k_records       64-byte hot records in leaf order (W = S^-1 R^T, mu, g0, index) and
 //                      the low float parts of W (48 B, read only by ill-conditioned hits)
-//   6. k_refit         bottom-up child boxes with one atomic counter per node
-//   7. k_collapse4     the 4-wide quantised tree: each binary internal node with up to four
+//   6. k_collapse4     the 4-wide quantised tree: each binary internal node with up to four
 //                      descendants, largest opened first (layout in ugp_internal.cuh)
 
 #include <math.h>
@@ -25,7 +24,7 @@ namespace {
 
 struct Layout {
   size_t prims, nodes, nodes4, wlo, persistent;
-  size_t aabb, keys0, keys1, vals0, vals1, parent, flags, bounds, sort, total;
+  size_t aabb, keys0, keys1, vals0, vals1, flags, bounds, sort, total;
 };
 
 __device__ __forceinline__ int f2o(float f) {
@@ -143,48 +142,8 @@ __global__ void k_morton(int64_t n, const float4* __restrict__ aabb, const int* 
   vals[i] = int32_t(i);
 }
 
-__device__ __forceinline__ int delta(const uint32_t* __restrict__ keys, int n, int i, int j) {
-  if (j < 0 || j >= n) return -1;
-  const uint32_t a = keys[i], b = keys[j];
-  if (a == b) return 32 + __clz(uint32_t(i) ^ uint32_t(j));
-  return __clz(a ^ b);
-}
-
-// One internal node per thread (n - 1 of them); node 0 is the root.
-__global__ void k_hierarchy(int n, const uint32_t* __restrict__ keys, int4* __restrict__ nodes,
-                            int32_t* __restrict__ parent_int, int32_t* __restrict__ parent_leaf) {
-  const int i = int(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n - 1) return;
-  const int d = (delta(keys, n, i, i + 1) - delta(keys, n, i, i - 1)) >= 0 ? 1 : -1;
-  const int dmin = delta(keys, n, i, i - d);
-  int lmax = 2;
-  while (delta(keys, n, i, i + lmax * d) > dmin) lmax <<= 1;
-  int l = 0;
-  for (int t = lmax >> 1; t >= 1; t >>= 1)
-    if (delta(keys, n, i, i + (l + t) * d) > dmin) l += t;
-  const int j = i + l * d;
-  const int dnode = delta(keys, n, i, j);
-  int s = 0;
-  for (int div = 2;; div <<= 1) {
-    const int t = (l + div - 1) / div;
-    if (delta(keys, n, i, i + (s + t) * d) > dnode) s += t;
-    if (t <= 1) break;
-  }
-  const int g = i + s * d + min(d, 0);
-  const int lo = min(i, j), hi = max(i, j);
-  int c0, c1;
-  if (lo == g) { c0 = ~g;      parent_leaf[g] = (i << 1) | 0; }
-  else         { c0 = g;       parent_int[g] = (i << 1) | 0; }
-  if (hi == g + 1) { c1 = ~(g + 1); parent_leaf[g + 1] = (i << 1) | 1; }
-  else             { c1 = g + 1;    parent_int[g + 1] = (i << 1) | 1; }
-  nodes[4 * i + 3] = make_int4(c0, c1, 0, 0);
-  if (i == 0) parent_int[0] = -1;
-}
-
-__global__ void k_single_root(int4* nodes, int32_t* parent_leaf, int32_t* parent_int) {
+__global__ void k_single_root(int4* nodes) {
   nodes[3] = make_int4(~0, kEmptyChild, 0, 0);
-  parent_leaf[0] = 0;
-  parent_int[0] = -1;
 }
 
 // Hot record of the primitive in leaf slot `slot` (layout in ugp_internal.cuh), plus the
@@ -227,44 +186,189 @@ __global__ void k_records(int64_t n, const int32_t* __restrict__ order, const fl
   wlo[3 * slot + 2] = l2;
 }
 
-__device__ __forceinline__ void store_child_box(float* node, int side, const float b[6]) {
-  float2* p = reinterpret_cast<float2*>(node + (side ? 6 : 0));
-  for (int k = 0; k < 3; ++k) p[k] = make_float2(b[2 * k], b[2 * k + 1]);
+// Binary radix tree over the sorted codes (Karras, HPG 2012) and its boxes. Node i has leaf i at one end of its
+// leaves, node 0 is the root. A block takes 256 leaves and the nodes of the same numbers.
+//   * A node whose leaves all lie in the block (its prefix is not shared by the leaf before the block or by the
+//     one behind it) finds its ends and its split by bisection, and its children's boxes from two windows
+//     of 2^k leaves each, which the block doubles in shared memory level by level: no node waits for another.
+//   * The others (about 1 in 25) are reached from below: the largest subtrees that lie in a block climb. Where two
+//     siblings meet both leave their box and far end for the split; the first to arrive stops, and the
+//     second, which knows the parent's leaves by then, writes it and goes on (Apetrei, CGVC 2014).
+// 5.5M primitives: nodes by one kernel 0.14 ms, boxes by climbing from every leaf with an atomic per node
+// 0.46, both by climbing with meetings in shared memory 0.52 (most lanes of a warp have stopped while one
+// climbs), now 0.28 and 0.07 for the climbers. Windows of all levels at once (47 KB) leave four blocks per SM,
+// windows of one level at a time cost twice the loads from shared memory: 0.36 and 0.32 in place of 0.28.
+constexpr int kTreeBlock = 256;
+constexpr unsigned kClimbBlocks = 8 * 152;
+
+// Where siblings of different blocks meet, and the subtrees that start from k_tree's blocks.
+struct Climb {
+  float4* meet;  // by split: the left child's box and first leaf, the right child's box and last leaf
+  int *flags;    // by split: children that have arrived
+  int *first, *last, *count;
+};
+// Length of the common prefix of the codes a, b of leaves p, q (equal codes: of their positions).
+__device__ __forceinline__ int prefix(uint32_t a, uint32_t b, int p, int q) {
+  return a == b ? 32 + __clz(uint32_t(p) ^ uint32_t(q)) : __clz(a ^ b);
+}
+__device__ __forceinline__ float united(int a, float x, float y) { return a < 3 ? fminf(x, y) : fmaxf(x, y); }
+__device__ __forceinline__ void leave_box(float4* meet, int split, int side, const float (&b)[6], int far) {
+  float4* m = meet + 4 * size_t(split) + 2 * side;
+  m[0] = make_float4(b[0], b[1], b[2], b[3]);
+  m[1] = make_float4(b[4], b[5], __int_as_float(far), 0.f);
+}
+// Node `id` over the leaves first .. last, its left child up to leaf `split`, with the children's boxes u and v.
+__device__ __forceinline__ void write_node(float4* nodes, int id, int first, int split, int last,
+                                           const float (&u)[6], const float (&v)[6]) {
+  float4* node = nodes + 4 * size_t(id);
+  node[0] = make_float4(u[0], u[1], u[2], u[3]);
+  node[1] = make_float4(u[4], u[5], v[0], v[1]);
+  node[2] = make_float4(v[2], v[3], v[4], v[5]);
+  reinterpret_cast<int4*>(node)[3] =
+      make_int4(first == split ? ~split : split, last == split + 1 ? ~(split + 1) : split + 1, 0, 0);
 }
 
-// Bottom-up boxes: each leaf writes its box into its parent, and the second of a node's
-// two children to arrive forms the union and continues upwards.
-__global__ void k_refit(int n, const int32_t* __restrict__ order, const float4* __restrict__ aabb,
-                        const int32_t* __restrict__ parent_int, const int32_t* __restrict__ parent_leaf,
-                        int* __restrict__ flags, float* __restrict__ nodes_f, float* __restrict__ root_box) {
-  const int slot = int(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (slot >= n) return;
-  const int i = order[slot];
-  const float4 lo = aabb[2 * i], hi = aabb[2 * i + 1];
-  float b[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
-  int ps = parent_leaf[slot];
-  while (true) {
-    const int p = ps >> 1, side = ps & 1;
-    store_child_box(nodes_f + 16 * size_t(p), side, b);
-    // the first of the two children to arrive leaves its box, the second goes on with the union
-    // (its own box is in registers, the sibling's is read once the flag says that it is there).
-    // One acquire-release atomic in place of two full fences, and 8-byte stores: 0.82 -> 0.47 ms of
-    // a build of 5.5M primitives
-    int seen;
-    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(seen) : "l"(flags + p) : "memory");
-    if (seen == 0) return;
-    const float2* o = reinterpret_cast<const float2*>(nodes_f + 16 * size_t(p) + (side ? 0 : 6));
-    const float2 o0 = __ldcg(o), o1 = __ldcg(o + 1), o2 = __ldcg(o + 2);
-    const float c[6] = {o0.x, o0.y, o1.x, o1.y, o2.x, o2.y};
-    for (int k = 0; k < 3; ++k) {
-      b[k] = fminf(b[k], c[k]);
-      b[3 + k] = fmaxf(b[3 + k], c[3 + k]);
+__global__ void __launch_bounds__(kTreeBlock) k_tree(int n, const uint32_t* __restrict__ keys,
+                                                     const int32_t* __restrict__ order,
+                                                     const float4* __restrict__ aabb, float4* __restrict__ nodes,
+                                                     float* __restrict__ root_box, Climb C) {
+  __shared__ uint32_t key[kTreeBlock + 2];  // of the leaves base - 1 .. base + kTreeBlock
+  __shared__ float win[4][6][kTreeBlock];   // boxes of the 2^k leaves from each on, four levels k; later the climbers
+  __shared__ int climbers, out;
+  const int tid = threadIdx.x, base = int(blockIdx.x) * kTreeBlock, end = min(base + kTreeBlock, n), i = base + tid;
+  for (int t = tid; t < kTreeBlock + 2; t += kTreeBlock) {
+    const int j = base - 1 + t;
+    key[t] = j >= 0 && j < n ? keys[j] : 0u;
+  }
+  if (tid == 0) climbers = 0;
+  float leaf[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+  if (i < n) {
+    const int p = order[i];
+    const float4 lo = aabb[2 * p], hi = aabb[2 * p + 1];
+    leaf[0] = lo.x; leaf[1] = lo.y; leaf[2] = lo.z; leaf[3] = hi.x; leaf[4] = hi.y; leaf[5] = hi.z;
+  }
+  for (int a = 0; a < 6; ++a) win[0][a][tid] = leaf[a];
+  __syncthreads();
+  auto delta = [&](int p, int q) {  // base - 1 <= p, q <= end; -1 outside of the scene
+    return p < 0 || q < 0 || p >= n || q >= n ? -1 : prefix(key[p - base + 1], key[q - base + 1], p, q);
+  };
+  int l = 0, r = 0, g = 0;
+  bool inside = false;
+  if (i < n - 1) {
+    const int dn = delta(i, i + 1), dp = delta(i, i - 1), d = dn > dp ? 1 : -1, dmin = min(dn, dp);
+    inside = !(delta(i, d > 0 ? end : base - 1) > dmin);
+    if (inside) {
+      // longer common prefix of (code, position) than `bits`: their difference is below 2^(63 - bits)
+      const uint32_t mine = key[tid + 1];
+      auto longer = [&](int q, unsigned long long limit) {
+        return ((unsigned long long)(mine ^ key[q - base + 1]) << 32 | uint32_t(i ^ q)) < limit;
+      };
+      const unsigned long long far = dmin < 0 ? ~0ull : 1ull << (63 - dmin);
+      int len = 0, s = 0;
+      for (int t = kTreeBlock / 2; t > 0; t >>= 1) {
+        const int q = i + (len + t) * d;
+        if (q >= base && q < end && longer(q, far)) len += t;
+      }
+      const int j = i + len * d;
+      const unsigned long long near = 1ull << (63 - delta(i, j));
+      for (int t = kTreeBlock / 2; t > 0; t >>= 1)
+        if (s + t <= len && longer(i + (s + t) * d, near)) s += t;
+      g = i + s * d + min(d, 0);
+      l = min(i, j);
+      r = max(i, j);
     }
-    ps = parent_int[p];
-    if (ps < 0) {
-      for (int k = 0; k < 6; ++k) root_box[k] = b[k];
-      return;
+  }
+  // a child's box from the windows of its size: at its first leaf and up to its last
+  float x[6], y[6], w[6];
+  for (int a = 0; a < 6; ++a) w[a] = leaf[a];
+  const int kl = inside ? 31 - __clz(g - l + 1) : -1, kr = inside ? 31 - __clz(r - g) : -1;
+  for (int k0 = 0; k0 < 8; k0 += 4) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k0 + k > 0) {
+        const int from = min(tid + (1 << (k0 + k - 1)), kTreeBlock - 1);
+        for (int a = 0; a < 6; ++a) w[a] = united(a, w[a], win[(k + 3) & 3][a][from]);
+        if (k == 0) __syncthreads();
+        for (int a = 0; a < 6; ++a) win[k][a][tid] = w[a];
+        __syncthreads();
+      }
     }
+    if (kl >= k0 && kl < k0 + 4)
+      for (int a = 0; a < 6; ++a)
+        x[a] = united(a, win[kl & 3][a][l - base], win[kl & 3][a][g - base + 1 - (1 << kl)]);
+    if (kr >= k0 && kr < k0 + 4)
+      for (int a = 0; a < 6; ++a)
+        y[a] = united(a, win[kr & 3][a][g + 1 - base], win[kr & 3][a][r - base + 1 - (1 << kr)]);
+    __syncthreads();
+  }
+  // a subtree climbs when its parent does not lie in the block
+  int(*own)[2] = reinterpret_cast<int(*)[2]>(&win[0][0][0]);
+  auto climbs = [&](int first, int last, const float (&u)[6]) {
+    const int dp = max(delta(first - 1, first), delta(last, last + 1));
+    if (delta(base - 1, first) < dp && delta(last, end) < dp) return;
+    const int side = delta(last, last + 1) == dp ? 0 : 1;
+    leave_box(C.meet, side ? first - 1 : last, side, u, side ? last : first);
+    int* c = own[atomicAdd(&climbers, 1)];  // disjoint subtrees of the block: at most 256
+    c[0] = first;
+    c[1] = last;
+  };
+  if (inside) {
+    write_node(nodes, i, l, g, r, x, y);
+    for (int a = 0; a < 6; ++a) x[a] = united(a, x[a], y[a]);
+    if (l == 0 && r == n - 1)
+      for (int a = 0; a < 6; ++a) root_box[a] = x[a];
+    else
+      climbs(l, r, x);
+  }
+  if (i < n) climbs(i, i, leaf);
+  __syncthreads();
+  if (tid == 0) out = atomicAdd(C.count, climbers);
+  __syncthreads();
+  if (tid < climbers) {
+    C.first[out + tid] = own[tid][0];
+    C.last[out + tid] = own[tid][1];
+  }
+}
+
+// The climbers, each by a thread. (In k_tree they kept their blocks for the two to four rounds of loads and
+// atomics that most climb, five times as long as the rest of the block's work: 0.48 ms in all.)
+__global__ void __launch_bounds__(kTreeBlock) k_climb(int n, const uint32_t* __restrict__ keys,
+                                                      float4* __restrict__ nodes, float* __restrict__ root_box,
+                                                      Climb C) {
+  const int count = *C.count;
+  auto delta = [&](int p, int q) { return p < 0 || q >= n ? -1 : prefix(keys[p], keys[q], p, q); };
+  for (int e = int(blockIdx.x) * kTreeBlock + threadIdx.x; e < count; e += int(gridDim.x) * kTreeBlock) {
+    int l = C.first[e], r = C.last[e];
+    int dl = delta(l - 1, l), dr = delta(r, r + 1);
+    float b[6];
+    bool left = true;  // the box for the parent is there
+    while (dl >= 0 || dr >= 0) {
+      const int side = dr > dl ? 0 : 1;  // left child or right
+      const int split = side ? l - 1 : r;
+      const float4* m = C.meet + 4 * size_t(split);
+      if (!left) leave_box(C.meet, split, side, b, side ? r : l);
+      // one acquire-release atomic in place of two full fences (boxes of 5.5M primitives: 0.82 -> 0.47 ms)
+      int seen;
+      asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(seen) : "l"(C.flags + split) : "memory");
+      if (seen == 0) break;
+      if (left) {
+        const float4 o0 = __ldcg(m + 2 * side), o1 = __ldcg(m + 2 * side + 1);
+        b[0] = o0.x; b[1] = o0.y; b[2] = o0.z; b[3] = o0.w; b[4] = o1.x; b[5] = o1.y;
+        left = false;
+      }
+      const float4 o0 = __ldcg(m + 2 - 2 * side), o1 = __ldcg(m + 3 - 2 * side);
+      const float c[6] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y};
+      if (side) l = __float_as_int(o1.z);
+      else r = __float_as_int(o1.z);
+      dl = delta(l - 1, l);
+      dr = delta(r, r + 1);
+      const int id = dl < 0 && dr < 0 ? 0 : (dr > dl ? r : l);  // a left child is node r, a right child node l
+      if (side) write_node(nodes, id, l, split, r, c, b);
+      else write_node(nodes, id, l, split, r, b, c);
+      for (int a = 0; a < 6; ++a) b[a] = united(a, b[a], c[a]);
+    }
+    if (dl < 0 && dr < 0)
+      for (int a = 0; a < 6; ++a) root_box[a] = b[a];
   }
 }
 
@@ -389,7 +493,6 @@ bool layout_for(int64_t n, Layout* L) {
   L->keys1 = off;      off = align256(off + N * 4);
   L->vals0 = off;      off = align256(off + N * 4);
   L->vals1 = off;      off = align256(off + N * 4);
-  L->parent = off;     off = align256(off + (ni + N) * 4);
   L->flags = off;      off = align256(off + ni * 4);
   L->sort = off;       off = align256(off + radix_sort_workspace(int64_t(N)));
   L->total = off;
@@ -457,9 +560,6 @@ extern "C" ugp_status ugp_build_bvh(const ugp_prims* prims, float cutoff_eps, vo
   uint32_t* k1 = reinterpret_cast<uint32_t*>(ws + L.keys1);
   int32_t* v0 = reinterpret_cast<int32_t*>(ws + L.vals0);
   int32_t* v1 = reinterpret_cast<int32_t*>(ws + L.vals1);
-  const size_t ni = n > 1 ? size_t(n - 1) : 1;
-  int32_t* parent_int = reinterpret_cast<int32_t*>(ws + L.parent);
-  int32_t* parent_leaf = parent_int + ni;
   int* flags = reinterpret_cast<int*>(ws + L.flags);
 
   const int T = 256;
@@ -475,7 +575,7 @@ extern "C" ugp_status ugp_build_bvh(const ugp_prims* prims, float cutoff_eps, vo
   int32_t* order = v0;
   if (n == 1) {
     UGP_CUDA_CHECK(cudaMemsetAsync(v0, 0, 4, st));
-    k_single_root<<<1, 1, 0, st>>>(nodes_i, parent_leaf, parent_int);
+    k_single_root<<<1, 1, 0, st>>>(nodes_i);
     k_single_refit<<<1, 1, 0, st>>>(aabb, nodes_f, root_box);
   } else {
     k_morton<<<G, T, 0, st>>>(n, aabb, bounds, k0, v0);
@@ -484,10 +584,17 @@ extern "C" ugp_status ugp_build_bvh(const ugp_prims* prims, float cutoff_eps, vo
     if (ss != UGP_OK) return ss;
     const bool in1 = (radix_sort_passes(30) & 1) != 0;
     order = in1 ? v1 : v0;
-    k_hierarchy<<<unsigned((n - 1 + T - 1) / T), T, 0, st>>>(int(n), in1 ? k1 : k0, nodes_i, parent_int, parent_leaf);
-    UGP_CUDA_CHECK(cudaGetLastError());
     UGP_CUDA_CHECK(cudaMemsetAsync(flags, 0, (n - 1) * 4, st));
-    k_refit<<<G, T, 0, st>>>(int(n), order, aabb, parent_int, parent_leaf, flags, nodes_f, root_box);
+    // the splits' boxes lie where the 4-wide nodes come to be
+    const Climb climb{reinterpret_cast<float4*>(ws + L.nodes4), flags, reinterpret_cast<int*>(in1 ? k0 : k1),
+                      in1 ? v0 : v1, bounds + 6};
+    const uint32_t* keys = in1 ? k1 : k0;
+    const unsigned tree_blocks = unsigned((n + kTreeBlock - 1) / kTreeBlock);
+    float4* nodes = reinterpret_cast<float4*>(ws + L.nodes);
+    k_tree<<<tree_blocks, kTreeBlock, 0, st>>>(int(n), keys, order, aabb, nodes, root_box, climb);
+    UGP_CUDA_CHECK(cudaGetLastError());
+    k_climb<<<tree_blocks < kClimbBlocks ? tree_blocks : kClimbBlocks, kTreeBlock, 0, st>>>(int(n), keys, nodes,
+                                                                                         root_box, climb);
     UGP_CUDA_CHECK(cudaGetLastError());
   }
   k_records<<<G, T, 0, st>>>(n, order, prims->mean3, prims->quat4, prims->scale3, prims->magnitude,

@@ -4,6 +4,7 @@
   is W to half an ulp, the pair to 2^-46 of its row's 1 / s (float64's own rounding, a few 2^-53 of
   the unit rotation, is far below), g0 to 1.5 ulp. Quaternions come with lengths from 1e-9 to 1e15 and
   scales over 20 decades, where products of the raw values would over- or underflow.
+* The binary nodes are the radix tree over the sorted codes, with exact boxes.
 * Every primitive is hit by the ray through its centre, whatever the shape of the tree: one, two
   and a few primitives (fewer children than a 4-wide node has), equal centres (ties in the code).
 """
@@ -101,3 +102,59 @@ def test_every_primitive_is_reached(ugp, n, spread):
     assert np.abs(T.cpu().numpy() - ref).max() <= 1e-5
     edge = np.abs(d2 - k2) < 1e-3
     assert (np.abs(cnt.cpu().numpy() - (d2 < k2).sum(1)) <= edge.sum(1)).all()
+
+
+@pytest.mark.parametrize("n", [2, 3, 128, 255, 256, 257, 512, 513, 30_011])
+@pytest.mark.parametrize("kind", ["spread", "ties"])
+def test_nodes_are_the_radix_tree_and_its_boxes(ugp, n, kind):
+    """The binary nodes equal the radix tree over (code, position), split at the highest differing bit and
+    numbered by the end of the leaves nearest the sibling; every box is the exact union of its leaves'."""
+    import torch
+    rng = np.random.Generator(np.random.Philox(n + (kind == "ties")))
+    mean = rng.uniform(-1, 1, (n, 3)).astype(np.float32)
+    if kind == "ties":   # a few positions, runs of equal codes longer than a block among them
+        mean = mean[np.minimum(rng.integers(0, 40, n), rng.integers(0, 40, n)) % n]
+    s = rng.uniform(0.01, 0.05, (n, 3)).astype(np.float32)
+    bvh = ugp.build_bvh(_dev(mean), _dev(scenes.random_quaternions(rng, n)), _dev(s), _dev(np.ones(n)))
+    torch.cuda.synchronize()
+    ws = bvh.workspace.cpu().numpy()
+    up = lambda x: (x + 255) // 256 * 256
+    rec = ws[: n * 64].view(np.float32).reshape(n, 4, 4)
+    node = ws[up(n * 64): up(n * 64) + (n - 1) * 64].view(np.float32).reshape(n - 1, 16)
+    child = node.view(np.int32)[:, 12:14]
+    assert (node[:, 14:] == 0).all()
+    leaf = np.zeros((n, 6), np.float32)
+    boxes = node[:, :12].reshape(-1, 6)
+    is_leaf = child.reshape(-1) < 0
+    assert sorted((~child.reshape(-1)[is_leaf]).tolist()) == list(range(n))
+    leaf[~child.reshape(-1)[is_leaf]] = boxes[is_leaf]
+    # codes of the leaves in order, from their boxes' centres between the means' extremes
+    lo, hi = mean.min(0), mean.max(0)
+    c = np.float32(0.5) * (leaf[:, :3] + leaf[:, 3:])
+    ext = hi - lo
+    t = np.where(ext > 0, (c - lo) / np.where(ext > 0, ext, 1), np.float32(0.5)).astype(np.float32)
+    t = np.clip(t * np.float32(1024), 0, 1023).astype(np.uint64)
+    code = np.zeros(n, np.uint64)
+    for b in range(10):
+        for a in range(3):
+            code |= ((t[:, a] >> np.uint64(b)) & np.uint64(1)) << np.uint64(3 * b + 2 - a)
+    assert (np.diff(code.astype(np.int64)) >= 0).all()
+    key = [int(x) << 32 | i for i, x in enumerate(code)]
+    arr = np.array(key, np.uint64)
+    todo = [(0, 0, n - 1)]
+    seen = 0
+    while todo:
+        i, l, r = todo.pop()
+        seen += 1
+        h = (key[l] ^ key[r]).bit_length() - 1
+        g = int(np.searchsorted(arr, np.uint64(key[r] >> h << h))) - 1
+        assert child[i].tolist() == [~g if l == g else g, ~(g + 1) if r == g + 1 else g + 1], (i, l, r)
+        for side, (p, q) in enumerate(((l, g), (g + 1, r))):
+            box = np.concatenate([leaf[p:q + 1, :3].min(0), leaf[p:q + 1, 3:].max(0)])
+            assert np.array_equal(node[i, 6 * side:6 * side + 6], box), (i, side)
+            if p < q:
+                todo.append(((g, g + 1)[side], p, q))
+    assert seen == n - 1
+    idx = rec[:, 3, 1].copy().view(np.int32)
+    for k in np.flatnonzero(np.diff(code.astype(np.int64)) == 0):   # equal codes keep the arrays' order
+        assert idx[k] < idx[k + 1]
