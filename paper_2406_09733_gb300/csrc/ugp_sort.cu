@@ -8,9 +8,11 @@
 //                  in earlier tiles) and the row's total;
 //   3. k_rs_scatter a tile's keys go to (keys of smaller digits) + (keys of this digit in earlier
 //                  tiles) + (keys of this digit earlier in the tile). Within the tile each warp
-//                  owns 1024 consecutive keys, counted per digit first; a warp then walks its
-//                  keys 32 at a time in order, and lanes holding the same digit rank themselves
-//                  by __match_any_sync, so equal keys keep their order (stable).
+//                  owns 512 consecutive keys and walks them 32 at a time in order; lanes holding
+//                  the same digit rank themselves by __match_any_sync, so equal keys keep their
+//                  order (stable). The tile is put in order in shared memory first and written out
+//                  from there: keys of a digit lie together, and a warp's store meets a few lines in
+//                  place of 32 (the four passes over 5.5M pairs: 0.26 -> 0.18 ms).
 // Passes alternate between the two buffers; the result is in buffer (passes & 1).
 #include "ugp_internal.cuh"
 
@@ -19,8 +21,8 @@ namespace {
 
 constexpr int kRsThreads = 256;
 constexpr int kRsWarps = kRsThreads / 32;
-constexpr int kRsPerWarp = 1024;
-constexpr int kTile = kRsWarps * kRsPerWarp;  // 8192 keys per tile
+constexpr int kRsPerWarp = 512, kRsPerLane = kRsPerWarp / 32;
+constexpr int kTile = kRsWarps * kRsPerWarp;  // 4096 keys per tile
 constexpr unsigned kFull = 0xffffffffu;
 
 __global__ void __launch_bounds__(kRsThreads) k_rs_hist(const uint32_t* __restrict__ keys, int64_t n, int shift,
@@ -83,53 +85,68 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_rows(uint32_t* __restrict__ h
   if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
-__global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const uint32_t* __restrict__ kin,
+// Three blocks per SM: 0.18 ms; two (101 registers) 0.22, four (64, spilled) 0.19.
+__global__ void __launch_bounds__(kRsThreads, 3) k_rs_scatter(const uint32_t* __restrict__ kin,
                                                             const int32_t* __restrict__ vin, int64_t n, int shift,
                                                             int tiles, const uint32_t* __restrict__ hist,
                                                             const uint32_t* __restrict__ totals,
                                                             uint32_t* __restrict__ kout, int32_t* __restrict__ vout) {
-  __shared__ uint32_t wbase[kRsWarps][256];
+  __shared__ uint32_t wbase[kRsWarps][256];  // keys of a digit a warp has met; then where its next one goes
+  __shared__ uint32_t skey[kTile], move[256];
+  __shared__ int32_t sval[kTile];
   __shared__ uint32_t ws[kRsWarps + 1];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int64_t first = int64_t(blockIdx.x) * kTile, wstart = first + int64_t(w) * kRsPerWarp + lane;
+  uint32_t key[kRsPerLane], rank[kRsPerLane];
+#pragma unroll
+  for (int r = 0; r < kRsPerLane; ++r) {
+    const int64_t idx = wstart + 32 * r;
+    key[r] = idx < n ? __ldg(kin + idx) : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < kRsWarps; ++k) wbase[k][tid] = 0u;
   // this tile's first position for digit tid: keys of smaller digits, then of digit tid in
   // earlier tiles
   uint32_t all;
   const uint32_t dpre = block_exclusive(totals[tid], ws, &all);
   const uint32_t gofs = dpre + hist[size_t(tid) * tiles + blockIdx.x];
-#pragma unroll
-  for (int k = 0; k < kRsWarps; ++k) wbase[k][tid] = 0u;
-  __syncthreads();
-  const int64_t wstart = int64_t(blockIdx.x) * kTile + int64_t(w) * kRsPerWarp;
-  for (int r = 0; r < kRsPerWarp; r += 32) {
-    const int64_t idx = wstart + r + lane;
-    if (idx < n) atomicAdd(&wbase[w][(__ldg(kin + idx) >> shift) & 255u], 1u);
-  }
-  __syncthreads();
-  {
-    uint32_t run = gofs;
-#pragma unroll
-    for (int k = 0; k < kRsWarps; ++k) {
-      const uint32_t c = wbase[k][tid];
-      wbase[k][tid] = run;
-      run += c;
-    }
-  }
-  __syncthreads();
   const unsigned below = (1u << lane) - 1u;
-  for (int r = 0; r < kRsPerWarp; r += 32) {
-    const int64_t idx = wstart + r + lane;
-    const bool valid = idx < n;
-    const uint32_t key = valid ? __ldg(kin + idx) : 0u;
-    const int d = valid ? int((key >> shift) & 255u) : 256 + lane;  // padding lanes match nobody
+#pragma unroll
+  for (int r = 0; r < kRsPerLane; ++r) {
+    const bool valid = wstart + 32 * r < n;
+    const int d = valid ? int((key[r] >> shift) & 255u) : 256 + lane;  // padding lanes match nobody
     const unsigned peers = __match_any_sync(kFull, d);
-    if (valid) {
-      const uint32_t pos = wbase[w][d] + __popc(peers & below);
-      kout[pos] = key;
-      vout[pos] = __ldg(vin + idx);
-    }
+    rank[r] = valid ? wbase[w][d] + __popc(peers & below) : 0u;
     __syncwarp();
     if (valid && (peers & below) == 0u) wbase[w][d] += __popc(peers);  // the digit's first lane
     __syncwarp();
+  }
+  __syncthreads();
+  uint32_t mine = 0u;
+#pragma unroll
+  for (int k = 0; k < kRsWarps; ++k) mine += wbase[k][tid];
+  uint32_t run = block_exclusive(mine, ws, &all);
+  move[tid] = gofs - run;
+#pragma unroll
+  for (int k = 0; k < kRsWarps; ++k) {
+    const uint32_t c = wbase[k][tid];
+    wbase[k][tid] = run;
+    run += c;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kRsPerLane; ++r)
+    if (wstart + 32 * r < n) {
+      const uint32_t pos = wbase[w][(key[r] >> shift) & 255u] + rank[r];
+      skey[pos] = key[r];
+      sval[pos] = __ldg(vin + wstart + 32 * r);
+    }
+  __syncthreads();
+  const int count = int(n - first < kTile ? n - first : kTile);
+  for (int e = tid; e < count; e += kRsThreads) {
+    const uint32_t k = skey[e], pos = move[(k >> shift) & 255u] + uint32_t(e);
+    kout[pos] = k;
+    vout[pos] = sval[e];
   }
 }
 

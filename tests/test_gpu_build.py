@@ -104,7 +104,7 @@ def test_every_primitive_is_reached(ugp, n, spread):
     assert (np.abs(cnt.cpu().numpy() - (d2 < k2).sum(1)) <= edge.sum(1)).all()
 
 
-@pytest.mark.parametrize("n", [2, 3, 128, 255, 256, 257, 512, 513, 30_011])
+@pytest.mark.parametrize("n", [2, 3, 128, 255, 256, 257, 512, 513, 4096, 4097, 30_011])
 @pytest.mark.parametrize("kind", ["spread", "ties"])
 def test_nodes_are_the_radix_tree_and_its_boxes(ugp, n, kind):
     """The binary nodes equal the radix tree over (code, position), split at the highest differing bit and
