@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(128) k_b_shade(BState S) {
         Lr = Lr + beta * f3(R.md.emission3[3 * k], R.md.emission3[3 * k + 1], R.md.emission3[3 * k + 2]);
       } else if (bounce < R.depth) {
         const Material M = load_material(R.md, k);
+        const SggxAxis axis = phase_axis(M);
         const float t = R.spawn == 1 ? P.tu[p] : P.ps.tsp[p];
         const float3 x = o + t * d, wo = -d;
         if (R.nee && L.has_quad && L.area > 0.f) {
@@ -294,7 +295,7 @@ __global__ void __launch_bounds__(128) k_b_shade(BState S) {
             const float Ue[6] = {Ua.x, Ua.y, Ua.z, Ua.w, Ub.x, Ub.y};
             const float3 f = phase_eval(M, wl, wo, Ue);
             if (f.x > 0.f || f.y > 0.f || f.z > 0.f) {
-              const float wm = mis_w(pl, phase_pdf_approx(M, wl, wo));
+              const float wm = mis_w(pl, phase_pdf_approx(M, axis, wl, wo));
               const float3 contrib = (wm / pl) * (beta * (f * L.Le));
               const int j = queue_append(&cw->shadow);
               S.sh.path[j] = p;
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(128) k_b_shade(BState S) {
         if (phase_sample(M, wo, U4, wi, wgt)) {
           beta = beta * wgt;
           if (beta.x > 0.f || beta.y > 0.f || beta.z > 0.f) {
-            P.ps.pdf_prev[p] = phase_pdf_approx(M, wi, wo);
+            P.ps.pdf_prev[p] = phase_pdf_approx(M, axis, wi, wo);
             P.ps.ox[p] = x.x; P.ps.oy[p] = x.y; P.ps.oz[p] = x.z;
             P.ps.dx[p] = wi.x; P.ps.dy[p] = wi.y; P.ps.dz[p] = wi.z;
             P.ps.br[p] = beta.x; P.ps.bg[p] = beta.y; P.ps.bb[p] = beta.z;

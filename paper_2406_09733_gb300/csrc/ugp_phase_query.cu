@@ -31,7 +31,7 @@ k_phase_query(int64_t n, const uint8_t* __restrict__ type, const float* __restri
   eval3[3 * i] = f.x;
   eval3[3 * i + 1] = f.y;
   eval3[3 * i + 2] = f.z;
-  pdf[i] = phase_pdf_approx(m, wi, wo);
+  pdf[i] = phase_pdf_approx(m, phase_axis(m), wi, wo);
   float V[4];
   for (int j = 0; j < 4; ++j) V[j] = us4[4 * i + j];
   float3 swi = f3(0.f, 0.f, 0.f), sw = f3(0.f, 0.f, 0.f);

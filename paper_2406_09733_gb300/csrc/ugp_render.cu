@@ -142,12 +142,14 @@ __global__ void __launch_bounds__(kFFBlock, kFew ? kFFBlocksWide : kFFBlocksPerS
   else scan_persistent(sm, src, scan_next);
 }
 
+constexpr int kShadeBlock = 128;
 template <bool kGuided>
-__global__ void __launch_bounds__(128) k_shade(MatDev mats, LightsDev L, uint2 key, int sample, int bounce, int max_depth,
+__global__ void __launch_bounds__(kShadeBlock) k_shade(MatDev mats, LightsDev L, uint2 key, int sample, int bounce, int max_depth,
                                                int nee, PathSoA ps, const int* __restrict__ q, const int* cnt,
                                                int* __restrict__ q_next, int* cnt_next, ShadowSoA sh, int* cnt_shadow,
                                                ShadowSoA she, int* cnt_shadow_e,
                                                int* dense_cnt, int* scan_next, GuidedShade gs, EmitterDev E) {
+  __shared__ float norms[kGuided ? kGLobes * kShadeBlock : 1];
   const bool em_on = emitters_on(E);
   const int count = load_count(cnt);
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // the extend and dense passes of this bounce have run
@@ -192,21 +194,15 @@ __global__ void __launch_bounds__(128) k_shade(MatDev mats, LightsDev L, uint2 k
       Lr = Lr + w * (beta * f3(mats.emission3[3 * k], mats.emission3[3 * k + 1], mats.emission3[3 * k + 2]));
     } else if (bounce < max_depth) {
       const Material M = load_material(mats, k);
+      const SggxAxis axis = phase_axis(M);
       const float t = ps.tsp[p];
       const float3 x = o + t * d, wo = -d;
       // the guide's share at this vertex: none where the base is glossier than min_rough (its
       // lobe is already sampled well; the guide, trained on radiance alone, would spread samples
       // outside it)
       const float al_v = kGuided && !guide_smooth(M, gs.min_rough) ? gs.alpha : 0.f;
-      float mix[kGuided ? kGOut : 1];
-      if (kGuided) {
-        const float4* m4 = reinterpret_cast<const float4*>(gs.mix + size_t(p) * kGOut);
-#pragma unroll
-        for (int j = 0; j < kGOut / 4; ++j) {
-          const float4 v = m4[j];
-          mix[4 * j] = v.x; mix[4 * j + 1] = v.y; mix[4 * j + 2] = v.z; mix[4 * j + 3] = v.w;
-        }
-      }
+      const VertexMixture<kShadeBlock> mix{gs.mix + (kGuided ? size_t(p) * kGOut : 0), norms + threadIdx.x};
+      if (kGuided) mix.prepare();
       if (nee && L.has_quad && L.area > 0.f) {
         const float4 Uy = rng(key, p, sample, bounce, 3);
         const float3 y = L.corner + Uy.x * L.e1 + Uy.y * L.e2;
@@ -220,8 +216,8 @@ __global__ void __launch_bounds__(128) k_shade(MatDev mats, LightsDev L, uint2 k
           const float Ue[6] = {Ua.x, Ua.y, Ua.z, Ua.w, Ub.x, Ub.y};
           const float3 f = phase_eval(M, wl, wo, Ue);
           if (f.x > 0.f || f.y > 0.f || f.z > 0.f) {
-            float ps_l = phase_pdf_approx(M, wl, wo);
-            if (kGuided) ps_l = al_v * mixture_pdf(mix, wl) + (1.f - al_v) * ps_l;
+            float ps_l = phase_pdf_approx(M, axis, wl, wo);
+            if (kGuided) ps_l = al_v * mix.pdf(wl) + (1.f - al_v) * ps_l;
             const float wm = mis_w(pl, ps_l);
             const float3 contrib = (wm / pl) * (beta * (f * L.Le));
             const int j = queue_append(cnt_shadow);
@@ -257,8 +253,8 @@ __global__ void __launch_bounds__(128) k_shade(MatDev mats, LightsDev L, uint2 k
           const float Ue[6] = {Ub.x, Ub.y, Ub.z, Ub.w, Uc.x, Uc.y};
           const float3 f = phase_eval(M, wl, wo, Ue);
           if (f.x > 0.f || f.y > 0.f || f.z > 0.f) {
-            float ps_l = phase_pdf_approx(M, wl, wo);
-            if (kGuided) ps_l = al_v * mixture_pdf(mix, wl) + (1.f - al_v) * ps_l;
+            float ps_l = phase_pdf_approx(M, axis, wl, wo);
+            if (kGuided) ps_l = al_v * mix.pdf(wl) + (1.f - al_v) * ps_l;
             const float3 c = f3(m0.w, m1.w, m2.w) - x;
             const float wm = mis_w(2.f * dot3(c, c) * pj, m3.x * ps_l);
             const float3 contrib = (wm * 0.5f * m3.x / (r2 * pj)) * (beta * (f * f3(m3.y, m3.z, m3.w)));
@@ -279,16 +275,16 @@ __global__ void __launch_bounds__(128) k_shade(MatDev mats, LightsDev L, uint2 k
         const float4 Us = rng(key, p, sample, bounce, 1);
         const float U4[4] = {Us.x, Us.y, Us.z, Us.w};
         sampled = phase_sample(M, wo, U4, wi, wgt);
-        if (sampled) pdf_s = phase_pdf_approx(M, wi, wo);
+        if (sampled) pdf_s = phase_pdf_approx(M, axis, wi, wo);
       } else {
         const float al = al_v;
         const float4 G = rng(key, p, sample, bounce, 2);
         if (G.y < al) {
-          wi = mixture_sample(mix, G.x, G.z, G.w);
+          wi = mix.sample(G.x, G.z, G.w);
           const float4 Ga = rng(key, p, sample, bounce, 6), Gb = rng(key, p, sample, bounce, 7);
           const float Ug[6] = {Ga.x, Ga.y, Ga.z, Ga.w, Gb.x, Gb.y};
           const float3 f = phase_eval(M, wi, wo, Ug);
-          pdf_s = al * mixture_pdf(mix, wi) + (1.f - al) * phase_pdf_approx(M, wi, wo);
+          pdf_s = al * mix.pdf(wi) + (1.f - al) * phase_pdf_approx(M, axis, wi, wo);
           sampled = pdf_s > 0.f;
           if (sampled) wgt = (1.f / pdf_s) * f;
         } else {
@@ -296,8 +292,8 @@ __global__ void __launch_bounds__(128) k_shade(MatDev mats, LightsDev L, uint2 k
           const float U4[4] = {Us.x, Us.y, Us.z, Us.w};
           float3 w0;
           if (phase_sample(M, wo, U4, wi, w0)) {
-            const float pt = phase_pdf_approx(M, wi, wo);
-            pdf_s = al * mixture_pdf(mix, wi) + (1.f - al) * pt;
+            const float pt = phase_pdf_approx(M, axis, wi, wo);
+            pdf_s = al * mix.pdf(wi) + (1.f - al) * pt;
             sampled = pdf_s > 0.f;
             if (sampled) wgt = (pt / pdf_s) * w0;
           }
@@ -648,7 +644,7 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
   const int g_cam = grid_for((const void*)k_camera, 256, n);
   const auto extend = n <= kFFFew && !stats ? k_extend<true> : k_extend<false>;
   const int g_ext = grid_for((const void*)extend, kFFBlock, 32 * n);  // down to one ray per warp
-  const int g_shade = guide ? grid_for((const void*)k_shade<true>, 128, n) : grid_for((const void*)k_shade<false>, 128, n);
+  const int g_shade = guide ? grid_for((const void*)k_shade<true>, kShadeBlock, n) : grid_for((const void*)k_shade<false>, kShadeBlock, n);
   // small images: groups of lanes per ray (the statistics count whole rays per lane)
   const bool few = n <= kTrFew && !stats;
   const int g_shadow = few ? tr_few_grid(n) : tr_grid(n);
@@ -681,11 +677,11 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
       }
       prof_begin(kStShade, st);
       if (guide)
-        k_shade<true><<<g_shade, 128, 0, st>>>(md, Ld, key, sample, b, params->max_depth, params->nee, ps, queue[cur],
+        k_shade<true><<<g_shade, kShadeBlock, 0, st>>>(md, Ld, key, sample, b, params->max_depth, params->nee, ps, queue[cur],
                                                 counts + cur, queue[nxt], counts + nxt, sh, counts + 2, she, counts + 4, dq.count + 2,
                                                 scan_next, gs, Em);
       else
-        k_shade<false><<<g_shade, 128, 0, st>>>(md, Ld, key, sample, b, params->max_depth, params->nee, ps,
+        k_shade<false><<<g_shade, kShadeBlock, 0, st>>>(md, Ld, key, sample, b, params->max_depth, params->nee, ps,
                                                  queue[cur], counts + cur, queue[nxt], counts + nxt, sh, counts + 2, she, counts + 4,
                                                  dq.count + 2, scan_next, gs, Em);
       prof_end(kStShade, st);
