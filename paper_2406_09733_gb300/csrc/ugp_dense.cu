@@ -112,6 +112,7 @@ struct WarpSmem {  // main pass: the two half-warps' slices
 struct WarpSmemBig {  // big pass: one ray per warp, its intervals in global memory
   static constexpr int kStack = kDStack;
   int stk[kStack];             // traversal stack
+  int leaves[96];              // leaves met and not yet handed on: fewer than 32 between steps
   unsigned long long bin[32];  // sub-bins, units of 2^-40
 };
 static_assert(kDCap >= kHalf && kBigCap >= kListCap, "capacities");
@@ -305,11 +306,13 @@ __device__ __forceinline__ void collect_one(const Grp<G>& g, const Iv& iv, const
 }
 
 // Warp-parallel traversal of the leaves whose boxes meet [lo, hi]; `leaf(slot)` is called by all
-// lanes together (slot < 0 for lanes without a leaf), twice per step.
+// lanes together, with 32 leaves at a time and once with what is left (slot < 0 for lanes without
+// one). A step meets a few leaves only: handed on as they were met, twice per step, the finish of a
+// 1920 x 1080 frame of 5.5M primitives took 52.9 ms, pooled 48.9.
 template <int kStack, class LeafFn>
-__device__ void warp_traverse(int* stk, const TraceScene& sc, const Ray& ray, float lo, float hi, int lane,
+__device__ void warp_traverse(int* stk, int* leaves, const TraceScene& sc, const Ray& ray, float lo, float hi, int lane,
                               uint8_t& st, unsigned& nn, LeafFn&& leaf) {
-  int size = 1;
+  int size = 1, held = 0;
   if (lane == 0) stk[0] = 0;
   __syncwarp();
   while (size > 0) {
@@ -354,11 +357,22 @@ __device__ void warp_traverse(int* stk, const TraceScene& sc, const Ray& ray, fl
       st = UGP_RAY_STACK_OVERFLOW;
       return;
     }
-    __syncwarp();
 #pragma unroll
-    for (int c = 0; c < 2; ++c) leaf((h[c] && ch[c] < 0) ? ~ch[c] : -1);
+    for (int c = 0; c < 2; ++c) {
+      const bool met = h[c] && ch[c] < 0;
+      const unsigned mask = __ballot_sync(kFull, met);
+      if (met) leaves[held + __popc(mask & ((1u << lane) - 1u))] = ~ch[c];
+      held += __popc(mask);
+    }
+    __syncwarp();
+    while (held >= 32) {
+      held -= 32;
+      leaf(leaves[held + lane]);
+    }
     __syncwarp();
   }
+  if (held > 0) leaf(lane < held ? leaves[lane] : -1);
+  __syncwarp();
 }
 
 // Per-ray inputs from slot j of the table.
@@ -497,7 +511,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_dense_big(TraceScene sc0, De
           collect_one(gw, iv, R.sc, R.ray, lo, hi, R.t0, R.t1, R.excl, e < R.nlist ? __ldg(R.list + e) : -1, n, np);
         }
       } else {
-        warp_traverse<WarpSmemBig::kStack>(W.stk, R.sc, R.ray, lo, hi, lane, st, nn, [&](int s) {
+        warp_traverse<WarpSmemBig::kStack>(W.stk, W.leaves, R.sc, R.ray, lo, hi, lane, st, nn, [&](int s) {
           collect_one(gw, iv, R.sc, R.ray, lo, hi, R.t0, R.t1, R.excl, s, n, np);
         });
       }
@@ -541,7 +555,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_dense_big(TraceScene sc0, De
             bin_one(e < R.nlist ? __ldg(R.list + e) : -1);
           }
         } else {
-          warp_traverse<WarpSmemBig::kStack>(W.stk, R.sc, R.ray, lo, hi, lane, st, nn, bin_one);
+          warp_traverse<WarpSmemBig::kStack>(W.stk, W.leaves, R.sc, R.ray, lo, hi, lane, st, nn, bin_one);
         }
         __syncwarp();
         if (st != UGP_RAY_OK) break;
