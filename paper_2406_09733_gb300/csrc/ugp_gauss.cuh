@@ -29,7 +29,12 @@ __device__ __forceinline__ Ray make_ray(float3 o, float3 d) {
   Ray r;
   r.o = o;
   r.d = d;
-  const float tiny = 1e-30f;
+  // A component that is zero against the others is given a size, so that a face beside the ray lies far beyond
+  // every segment: 1e-20 of the largest one moves the ray by far less than any box is widened, and keeps the
+  // node test finite (2^15 grid steps over this size, node4_test) for nodes up to 2.6e16 |d| wide. At a fixed 1e-30
+  // that ended at 2.1e6, and such rays missed every child of a wider root. The floor, for very short d,
+  // still allows 5e8.
+  const float tiny = fmaxf(1e-20f * fmaxf(fmaxf(fabsf(d.x), fabsf(d.y)), fabsf(d.z)), 2e-28f);
   r.inv.x = 1.f / (fabsf(d.x) > tiny ? d.x : copysignf(tiny, d.x));
   r.inv.y = 1.f / (fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y));
   r.inv.z = 1.f / (fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z));
@@ -366,7 +371,8 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
 // The ray's direction signs pick, once per node, which face of each axis is met first, so a
 // child's entry and exit are a three-way max and min (the same values as the min/max pairs). The
 // faces come with an offset of 2^15 (byte_f), so the line's constant is rounded at that size, an
-// error of up to 2^-9 grid steps, which the faces' margin of 2^-7 steps covers (k_collapse4). One
+// error of up to 2^-9 grid steps, which the faces' margin of 2^-7 steps covers (k_collapse4). The line's constant
+// must stay finite: make_ray bounds inv for that. One
 // instruction less per face than taking the offset away from each: 1,000,003 light-sample rays in a
 // 1M-primitive room 3.01 -> 2.93 ms.
 __device__ __forceinline__ unsigned node4_test(const uint4* __restrict__ n4, int node, const Ray& r, float tmin,
