@@ -373,7 +373,8 @@ __global__ void __launch_bounds__(kTreeBlock) k_climb(int n, const uint32_t* __r
 }
 
 // One 4-wide node per binary internal node: its children, of which the internal one with the largest
-// surface is replaced by its own two until there are four. (Every binary node gets one, as any of them
+// surface is replaced by its own two until there are four, the other child before a grandchild of the same size
+// (equal boxes, as of primitives in one place, then give a tree of half the depth). (Every binary node gets one, as any of them
 // may be a child. With two fixed levels a child that is a leaf left a slot empty, and depths had to be
 // found first by eight launches: rebuilding 5.5M primitives took 2.47 ms against 2.15, light-sample
 // rays in a 1M-primitive room 2.94 ms per million against 2.75, free flights 7.04 against 6.94.) Boxes are quantised outwards to
@@ -402,13 +403,15 @@ __global__ void __launch_bounds__(256) k_collapse4(int n_int, const float4* __re
   int m = ref[1] == kEmptyChild ? 1 : 2;  // one only for the root of a one-primitive tree
   if (m == 2) {
     if (area[0] >= 0.f || area[1] >= 0.f) {
-      if (area[0] >= area[1]) open(ref[0], 0, 2);
+      const bool left = area[0] >= area[1];
+      if (left) open(ref[0], 0, 2);
       else open(ref[1], 1, 2);
       m = 3;
       const float big = fmaxf(area[0], fmaxf(area[1], area[2]));
       if (big >= 0.f) {
-        if (area[0] == big) open(ref[0], 0, 3);
-        else if (area[1] == big) open(ref[1], 1, 3);
+        const int c = (left ? area[1] : area[0]) == big ? (left ? 1 : 0) : (area[2] == big ? 2 : (left ? 0 : 1));
+        if (c == 0) open(ref[0], 0, 3);
+        else if (c == 1) open(ref[1], 1, 3);
         else open(ref[2], 2, 3);
         m = 4;
       }

@@ -265,8 +265,8 @@ static __device__ void pooled_leaf(FFSmem<kStack>& sm, const OwnerRay& w, int sl
 // zero before the launch. The node step is written out in the loop with the traversal state in
 // plain locals; kept in this form, the compiler holds the state in registers across the refill
 // branch (the same steps written as helper functions over ScanState ran 1.4x slower).
-// With kStack < kFFStack the stack's top entries beyond it are kept in local memory (few rays get there):
-// six blocks of the scan then share an SM instead of five, 6.94 -> 6.79 ms for 2^20 camera and bounce rays
+// The stack's entries beyond kStack are kept in local memory (few rays get there): with 26 in shared memory in
+// place of 36, six blocks of the scan share an SM instead of five, 6.94 -> 6.79 ms for 2^20 camera and bounce rays
 // through a 1M-primitive room.
 template <class Src, int kStack>
 __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
@@ -279,8 +279,7 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
   const int used = rays_per_warp(n, int64_t(gridDim.x) * (kFFBlock / 32));
   const int refill_at = max(1, min(kRefill, used / 4));
   bool busy = false, exhausted = lane >= used, tdone = false;
-  constexpr int kDeep = kFFStack - kStack;
-  int deep[kDeep > 0 ? kDeep : 1];
+  int deep[kStackMax - kStack];
   int node = 0, sp = 0, jc = kB, nq = 0;
   float lo = 0.f, hi = 0.f, L = 0.f, target = 0.f, limit = 0.f;
   for (;;) {
@@ -469,7 +468,7 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
         tdone = true;
         nq = 0;
       } else if (nk > 0) {
-        if (sp + nk - 1 > kFFStack) {
+        if (sp + nk - 1 > kStackMax) {
           c.st = UGP_RAY_STACK_OVERFLOW;
           tdone = true;
           nq = 0;
@@ -478,7 +477,7 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
 #pragma unroll
           for (int k = 3; k >= 1; --k)
             if (rk[k] >= 0) {
-              if (kDeep == 0 || sp < kStack) sm.stk[sp][c.tid] = rk[k];
+              if (sp < kStack) sm.stk[sp][c.tid] = rk[k];
               else deep[sp - kStack] = rk[k];
               ++sp;
             }
@@ -488,7 +487,7 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
         tdone = true;
       } else {
         --sp;
-        node = kDeep == 0 || sp < kStack ? sm.stk[sp][c.tid] : deep[sp - kStack];
+        node = sp < kStack ? sm.stk[sp][c.tid] : deep[sp - kStack];
       }
     }
   }
@@ -509,6 +508,8 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
   const unsigned below_me = (1u << lane) - 1u, above_me = lane == 31 ? 0u : ~0u << (lane + 1);
   const bool head = lane == gbase;
   auto at = [&](int i) -> int& { return sm.stk[i >> lg][gtid + (i & (gsize - 1))]; };
+  const int grows = kFFStack << lg;    // the group's stack in shared memory; its first lane holds what lies above
+  int deep[kStackMax - kFFStack];
   const int n = src.count();
   const int groups = 32 >> lg;
   const int used = min(groups, rays_per_warp(n, int64_t(gridDim.x) * (kFFBlock / 32)));
@@ -684,12 +685,15 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
         if (jc < kB) limit = bin_edge(lo, hi, L, jc + 1);
       }
     } else {
-      // ---- node step: a node per lane from the top of the group's stack, all lanes together (one once
-      // the stack is half full: it then grows by three a level, as a single lane's does)
-      const int k0 = lane - gbase, m = busy && !tdone ? min(sp, sp > (kFFStack << lg) / 2 ? 1 : gsize) : 0;
+      // ---- node step: a node per lane from the top of the group's stack, all lanes together (one, by the first lane,
+      // once the stack is half full: it then grows by three a level, as a single lane's does)
+      const int k0 = lane - gbase, m = busy && !tdone ? min(sp, sp > grows / 2 ? 1 : gsize) : 0;
       const bool act = k0 < m;
       int node = 0;
-      if (act) node = at(sp - 1 - k0);
+      if (act) {
+        const int i = sp - 1 - k0;
+        node = i < grows ? at(i) : deep[i - grows];
+      }
       sp -= m;
       float tk[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
       int rk[4] = {-1, -1, -1, -1};
@@ -724,7 +728,7 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
       const int pushed = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
       const int base = sp + __popc(b0 & above_me) + 2 * __popc(b1 & above_me) + 4 * __popc(b2 & above_me);
       const bool g_bad = (__ballot_sync(kFull, bad) & glanes) != 0u;
-      const bool full = sp + pushed > kFFStack << lg;
+      const bool full = sp + pushed > grows + (kStackMax - kFFStack);
       if (m > 0 && (g_bad || full)) {
         st = g_bad ? UGP_RAY_BAD_NODE : UGP_RAY_STACK_OVERFLOW;
         tdone = true;
@@ -732,7 +736,11 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
       } else if (m > 0) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          if (rk[k] >= 0) at(base + nk - 1 - k) = rk[k];  // hits are sorted first; the nearest on top
+          if (rk[k] >= 0) {  // hits are sorted first; the nearest on top
+            const int i = base + nk - 1 - k;
+            if (i < grows) at(i) = rk[k];
+            else deep[i - grows] = rk[k];
+          }
         sp += pushed;
         if (sp == 0) tdone = true;
       }

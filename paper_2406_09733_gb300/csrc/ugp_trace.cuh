@@ -6,13 +6,18 @@
 namespace ugp {
 
 constexpr int kTrBlock = 128;      // transmittance: threads per block
-constexpr int kTrStack = 48;       // transmittance: traversal stack depth
+constexpr int kTrStack = 48;       // transmittance: rows of shared memory for stack and held-back primitives
 constexpr int kTrBlocksPerSM = 8;  // transmittance: resident blocks per SM (24 KB shared, <= 64 registers)
 constexpr int kFFBlock = 128;      // free flight: threads per block of the scan
-constexpr int kFFStack = 36;       // free flight: traversal stack depth (4-wide nodes)
-constexpr int kFFShort = 26;       // of it in shared memory where six blocks of the scan share an SM
+constexpr int kFFStack = 36;       // free flight: rows of the traversal stack in shared memory
+constexpr int kFFShort = 26;       // the same where six blocks of the scan share an SM
 constexpr int kFFBlocksPerSM = 6;  // free flight: resident scan blocks per SM (37 KB shared, <= 80 registers)
 constexpr int kFFBlocksWide = 5;   // the same for scans with more state (groups, a scene per ray; 42 KB, <= 102)
+// Entries that a traversal of the 4-wide tree can need at most. A step down a path is at least one level of the binary
+// tree over 30-bit codes and, for equal codes, 30-bit positions (60 levels), and leaves up to three children on the
+// stack. Rooms need 28; scenes whose sizes span decades around one place need 40 to 80. What lies
+// above the rows in shared memory is kept in local memory, which only rays that get there touch.
+constexpr int kStackMax = 3 * 60;
 constexpr int kB = 32;             // free flight: bins of the scan
 constexpr int kTrWarps = 152 * kTrBlocksPerSM * kTrBlock / 32;  // warps of the transmittance a GB300 holds
 

@@ -38,7 +38,8 @@ static_assert(kTrLeafQ < 16, "queue lengths are summed from four bit planes");
 //
 // With kGroup, 1 << lg neighbouring lanes share a ray (its arguments are the same on all of them): the
 // stack columns of a group are one stack, and a node step takes a node per lane from its top, nearest in
-// the group's first lane. A launch of few rays is bound by the chain of dependent steps of its longest
+// the group's first lane. (Above half of the rows, which 4 lanes have 76 of, the stack holds at most 3 lanes + kStackMax
+// entries: those of the last step of all lanes, then three a level of one path.) A launch of few rays is bound by the chain of dependent steps of its longest
 // ray, and this shortens the chain, where spreading the rays over the warps left most lanes idle (figures at
 // tr_group).
 template <bool kGroup, bool kOneScene, class P>
@@ -50,12 +51,15 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
   const unsigned below_me = (1u << lane) - 1u;
   int sp = 0, node = 0, nq = 0;
   bool tdone = !(live && sc.n_prims > 0 && t0 < t_far), done = tdone;
-  int* lq = stk + (kTrStack - kTrLeafQ) * stride;
+  constexpr int kRows = kTrStack - kTrLeafQ;  // of the stack in shared memory
+  int* lq = stk + kRows * stride;
+  int deep[kStackMax - kRows];
   // the group: its first lane, its lanes, its stack (entry i in row i >> lg of column i & (lanes - 1))
   const int gsize = kGroup ? 1 << lg : 1, gbase = lane & ~(gsize - 1);
   const unsigned glanes = (gsize == 32 ? ~0u : (1u << gsize) - 1u) << gbase;
   int* const gstk = stk - (lane - gbase);
   auto at = [&](int i) -> int& { return gstk[(i >> lg) * stride + (i & (gsize - 1))]; };
+  const int grows = kRows << lg;  // the group's entries in shared memory
   if (kGroup) {
     if (lane == gbase) at(0) = 0;
     sp = 1;  // entries of the group's stack (with a lane per ray: below the current node)
@@ -112,11 +116,14 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
         }
       }
     } else if (kGroup) {
-      // ---- node step of groups: all lanes together (one node once the stack is half full: it then
-      // grows by three a level, as a single lane's does)
-      const int k0 = lane - gbase, m = tdone || done ? 0 : min(sp, sp > ((kTrStack - kTrLeafQ) << lg) / 2 ? 1 : gsize);
+      // ---- node step of groups: all lanes together (one node, by the first lane, once the stack is half full: it
+      // then grows by three a level, as a single lane's does, and may go on in that lane's local memory)
+      const int k0 = lane - gbase, m = tdone || done ? 0 : min(sp, sp > grows / 2 ? 1 : gsize);
       const bool act = k0 < m;
-      if (act) node = at(sp - 1 - k0);
+      if (act) {
+        const int i = sp - 1 - k0;
+        node = i < grows ? at(i) : deep[i - grows];
+      }
       sp -= m;
       float tk[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
       int rk[4] = {-1, -1, -1, -1};
@@ -153,7 +160,7 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
       const int pushed = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
       const int base = sp + __popc(b0 & above) + 2 * __popc(b1 & above) + 4 * __popc(b2 & above);
       const bool g_bad = (__ballot_sync(mask, bad) & glanes) != 0u;
-      const bool full = sp + pushed > (kTrStack - kTrLeafQ) << lg;
+      const bool full = sp + pushed > grows + (kStackMax - kRows);
       if (m > 0 && (g_bad || full)) {
         ts.st = g_bad ? UGP_RAY_BAD_NODE : UGP_RAY_STACK_OVERFLOW;
         tdone = true;
@@ -161,7 +168,11 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
       } else if (m > 0) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          if (rk[k] >= 0) at(base + nk - 1 - k) = rk[k];  // hits are sorted first
+          if (rk[k] >= 0) {  // hits are sorted first
+            const int i = base + nk - 1 - k;
+            if (i < grows) at(i) = rk[k];
+            else deep[i - grows] = rk[k];
+          }
         sp += pushed;
         if (sp == 0) tdone = true;
       }
@@ -207,10 +218,23 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
           tdone = true;
           nq = 0;
         } else if (nk > 0) {
-          if (sp + nk - 1 > kTrStack - kTrLeafQ) {
-            ts.st = UGP_RAY_STACK_OVERFLOW;
-            tdone = true;
-            nq = 0;
+          // rare, and apart from the plain pushes: 1,000,003 light-sample rays in a 1M-primitive room take 2.74 ms
+          // (2.75 with no rows beyond shared memory), with a comparison at each push 2.82
+          if (sp + nk - 1 > kRows) {
+            if (sp + nk - 1 > kStackMax) {
+              ts.st = UGP_RAY_STACK_OVERFLOW;
+              tdone = true;
+              nq = 0;
+            } else {
+#pragma unroll
+              for (int k = 3; k >= 1; --k)
+                if (rk[k] >= 0) {
+                  if (sp < kRows) stk[sp * stride] = rk[k];
+                  else deep[sp - kRows] = rk[k];
+                  ++sp;
+                }
+              node = rk[0];
+            }
           } else {
 #pragma unroll
             for (int k = 3; k >= 1; --k)
@@ -224,7 +248,8 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
           tdone = true;
         } else {
           --sp;
-          node = stk[sp * stride];
+          if (__builtin_expect(sp >= kRows, 0)) node = deep[sp - kRows];
+          else node = stk[sp * stride];
         }
       }
     }
