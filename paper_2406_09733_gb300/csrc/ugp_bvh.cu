@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(256) k_collapse4(int n_int, const float4* __re
       qlo[a] |= uint32_t(ql) << (8 * c);
       qhi[a] |= uint32_t(qh) << (8 * c);
     }
-    // an empty child slot gets an inverted box (low face 255, high face 0) that no ray enters,
-    // so the node test needs no separate check for it
+    // an empty child slot gets an inverted box (low face 255, high face 0), which a ray enters only where the
+    // whole node is below the node test's slack
 #pragma unroll
     for (int c = 1; c < 4; ++c)
       if (c >= m) qlo[a] |= 255u << (8 * c);

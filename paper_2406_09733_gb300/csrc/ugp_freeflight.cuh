@@ -443,17 +443,19 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
       ++c.n_nodes;
       float tk[4];
       int rk[4];
-      int nk = 0;
+      int nk = 0, inv = 0;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 3; k >= 0; --k) {
         tk[k] = INFINITY;
         rk[k] = -1;
         if (!((hm >> k) & 1u)) continue;
         // a primitive's slot is checked here (its record is loaded by slot); a child node's
         // index is checked when it is visited
-        if (ch[k] < 0 && unsigned(~ch[k]) >= unsigned(src.scene().n_prims)) c.st = UGP_RAY_BAD_NODE;
-        if (c.st != UGP_RAY_OK) continue;
         if (ch[k] < 0) {
+          if (unsigned(~ch[k]) >= unsigned(src.scene().n_prims)) {
+            inv = ch[k];
+            continue;
+          }
           ++c.n_prims;
           sm.lq[nq][c.tid] = ~ch[k];  // nq <= kLeafQ - 4 here: a node adds at most four
           ++nq;
@@ -464,6 +466,7 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
         }
       }
       sort4(tk, rk);
+      if (!valid_ref(inv)) c.st = UGP_RAY_BAD_NODE;
       if (c.st != UGP_RAY_OK) {
         tdone = true;
         nq = 0;
@@ -698,18 +701,18 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
       float tk[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
       int rk[4] = {-1, -1, -1, -1};
       int nk = 0;
-      bool bad = act && unsigned(node) >= unsigned(sc.n_nodes);
-      if (act && !bad) {
+      int inv = act && unsigned(node) >= unsigned(sc.n_nodes) ? -1 : 0;  // see valid_ref
+      if (act && inv == 0) {
         float en[4];
         int ch[4];
         const unsigned hm = node4_test(sc.nodes4, node, ray, lo, limit, en, ch);
         ++n_nodes;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 3; k >= 0; --k) {
           if (!((hm >> k) & 1u)) continue;
           if (ch[k] < 0) {
             if (unsigned(~ch[k]) >= unsigned(sc.n_prims)) {
-              bad = true;
+              inv = ch[k];
               continue;
             }
             ++n_prims;
@@ -727,7 +730,7 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
                      b2 = __ballot_sync(kFull, (nk & 4) != 0) & glanes;
       const int pushed = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
       const int base = sp + __popc(b0 & above_me) + 2 * __popc(b1 & above_me) + 4 * __popc(b2 & above_me);
-      const bool g_bad = (__ballot_sync(kFull, bad) & glanes) != 0u;
+      const bool g_bad = (__ballot_sync(kFull, !valid_ref(inv)) & glanes) != 0u;
       const bool full = sp + pushed > grows + (kStackMax - kFFStack);
       if (m > 0 && (g_bad || full)) {
         st = g_bad ? UGP_RAY_BAD_NODE : UGP_RAY_STACK_OVERFLOW;

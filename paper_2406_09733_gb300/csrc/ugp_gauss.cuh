@@ -366,7 +366,11 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
 
 // Slab test of the four children of a 4-wide quantised node (layout in ugp_internal.cuh)
 // against [tmin, tmax]: returns the mask of children hit and writes their references and entry
-// distances. Child c's face along axis a is o_a + q 2^e_a, so its ray distance is
+// distances. An empty slot, whose box is inverted, is hit only where the whole node is smaller than the slack
+// for rounding (4e-7 of the distance); valid_ref tells it from a reference that is none. The callers look at
+// the slots from the last to the first, and empty ones come last, so the reference they keep for that is a
+// wrong one if there is any. (A mask of the slots in use, applied here, cost the transmittance 2.7%, a
+// second comparison in the callers' loops 0.8%; this nothing.) Child c's face along axis a is o_a + q 2^e_a, so its ray distance is
 // q (2^e_a inv_a) + (o_a - ray.o_a) inv_a: two products per axis and node, one fma per face.
 // The ray's direction signs pick, once per node, which face of each axis is met first, so a
 // child's entry and exit are a three-way max and min (the same values as the min/max pairs). The
@@ -402,10 +406,14 @@ __device__ __forceinline__ unsigned node4_test(const uint4* __restrict__ n4, int
     const float th = fminf(min3f(fmaf(byte_f(fx, c), ax, bx), fmaf(byte_f(fy, c), ay, by), fmaf(byte_f(fz, c), az, bz)),
                            tmax);
     en[c] = tl;
-    if (tl <= th + 4e-7f * fabsf(th)) hit |= 1u << c;  // never for an empty slot (inverted box)
+    if (tl <= th + 4e-7f * fabsf(th)) hit |= 1u << c;
   }
   return hit;
 }
+
+// Whether `inv`, the last reference of a node step that was no primitive's and no node's (0: none), is an empty
+// slot's or none.
+__device__ __forceinline__ bool valid_ref(int inv) { return unsigned(inv) <= unsigned(kEmptyChild); }
 
 // Orders (t, ref) pairs of the children hit by entry distance (misses last), a sorting network
 // on four entries.

@@ -39,9 +39,9 @@ constexpr int kEmptyChild = INT32_MIN;
 //        index, < 0 and != kEmptyChild the leaf holding primitive slot ~child, kEmptyChild none.
 // Child c's box along axis a is [o_a + lo_a(c) 2^e_a, o_a + hi_a(c) 2^e_a]; the faces are rounded
 // outwards with a margin of 2^-7 grid steps, so the quantised box contains the exact one by more than
-// the node test's rounding. An empty slot's box is inverted
-// (lo = 255, hi = 0 on every axis), so no ray enters it. A 4-wide node sits at the index of its
-// binary node (the nodes that were absorbed are never read).
+// the node test's rounding. An empty slot's box is inverted (lo = 255, hi = 0 on every axis); a ray enters it only
+// where the whole node is smaller than the node test's slack, and takes it for a miss. The empty slots are
+// the last ones. A 4-wide node sits at the index of its binary node (the nodes that were absorbed are never read).
 constexpr int kNode4U4 = 4;
 
 }  // namespace ugp

@@ -128,18 +128,18 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
       float tk[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
       int rk[4] = {-1, -1, -1, -1};
       int nk = 0;
-      bool bad = act && unsigned(node) >= unsigned(sc.n_nodes);
-      if (act && !bad) {
+      int inv = act && unsigned(node) >= unsigned(sc.n_nodes) ? -1 : 0;  // see valid_ref
+      if (act && inv == 0) {
         float en[4];
         int ch[4];
         const unsigned hm = node4_test(sc.nodes4, node, ray, t0, t_far, en, ch);
         ++ts.n_nodes;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 3; k >= 0; --k) {
           if (!((hm >> k) & 1u)) continue;
           if (ch[k] < 0) {
             if (unsigned(~ch[k]) >= unsigned(sc.n_prims)) {
-              bad = true;
+              inv = ch[k];
               continue;
             }
             ++ts.n_prims;
@@ -159,7 +159,7 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
       const unsigned above = lane == 31 ? 0u : ~0u << (lane + 1);
       const int pushed = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
       const int base = sp + __popc(b0 & above) + 2 * __popc(b1 & above) + 4 * __popc(b2 & above);
-      const bool g_bad = (__ballot_sync(mask, bad) & glanes) != 0u;
+      const bool g_bad = (__ballot_sync(mask, !valid_ref(inv)) & glanes) != 0u;
       const bool full = sp + pushed > grows + (kStackMax - kRows);
       if (m > 0 && (g_bad || full)) {
         ts.st = g_bad ? UGP_RAY_BAD_NODE : UGP_RAY_STACK_OVERFLOW;
@@ -190,9 +190,9 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
         float tk[4];
         int rk[4];
         int nk = 0;
-        bool bad = false;
+        int inv = 0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 3; k >= 0; --k) {
           tk[k] = INFINITY;
           rk[k] = -1;
           if (!((hm >> k) & 1u)) continue;
@@ -200,7 +200,7 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
             // a primitive's slot is checked here (its record is loaded by slot); a child node's
             // index is checked when it is visited
             if (unsigned(~ch[k]) >= unsigned(sc.n_prims)) {
-              bad = true;
+              inv = ch[k];
               continue;
             }
             ++ts.n_prims;
@@ -213,7 +213,7 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
           }
         }
         if (P::kNearFirst || rk[0] < 0) sort4(tk, rk);  // at least, the first is one that was hit
-        if (bad) {
+        if (!valid_ref(inv)) {
           ts.st = UGP_RAY_BAD_NODE;
           tdone = true;
           nq = 0;
