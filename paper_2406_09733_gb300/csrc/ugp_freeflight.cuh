@@ -471,17 +471,27 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
         tdone = true;
         nq = 0;
       } else if (nk > 0) {
-        if (sp + nk - 1 > kStackMax) {
-          c.st = UGP_RAY_STACK_OVERFLOW;
-          tdone = true;
-          nq = 0;
+        // the farther children go on the stack, farthest first, so the nearer pop first
+        if (sp + nk - 1 > kStack) {  // rare
+          if (sp + nk - 1 > kStackMax) {
+            c.st = UGP_RAY_STACK_OVERFLOW;
+            tdone = true;
+            nq = 0;
+          } else {
+#pragma unroll
+            for (int k = 3; k >= 1; --k)
+              if (rk[k] >= 0) {
+                if (sp < kStack) sm.stk[sp][c.tid] = rk[k];
+                else deep[sp - kStack] = rk[k];
+                ++sp;
+              }
+            node = rk[0];
+          }
         } else {
-          // the farther children go on the stack, farthest first, so the nearer pop first
 #pragma unroll
           for (int k = 3; k >= 1; --k)
             if (rk[k] >= 0) {
-              if (sp < kStack) sm.stk[sp][c.tid] = rk[k];
-              else deep[sp - kStack] = rk[k];
+              sm.stk[sp][c.tid] = rk[k];
               ++sp;
             }
           node = rk[0];
@@ -490,7 +500,8 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
         tdone = true;
       } else {
         --sp;
-        node = sp < kStack ? sm.stk[sp][c.tid] : deep[sp - kStack];
+        if (__builtin_expect(sp >= kStack, 0)) node = deep[sp - kStack];
+        else node = sm.stk[sp][c.tid];
       }
     }
   }
@@ -694,8 +705,8 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
       const bool act = k0 < m;
       int node = 0;
       if (act) {
-        const int i = sp - 1 - k0;
-        node = i < grows ? at(i) : deep[i - grows];
+        if (__builtin_expect(sp > grows, 0)) node = deep[sp - 1 - grows];
+        else node = at(sp - 1 - k0);
       }
       sp -= m;
       float tk[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
@@ -737,13 +748,19 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
         tdone = true;
         nq = 0;
       } else if (m > 0) {
+        if (__builtin_expect(sp + pushed > grows, 0)) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (rk[k] >= 0) {  // hits are sorted first; the nearest on top
-            const int i = base + nk - 1 - k;
-            if (i < grows) at(i) = rk[k];
-            else deep[i - grows] = rk[k];
-          }
+          for (int k = 0; k < 4; ++k)
+            if (rk[k] >= 0) {  // hits are sorted first; the nearest on top
+              const int i = base + nk - 1 - k;
+              if (i < grows) at(i) = rk[k];
+              else deep[i - grows] = rk[k];
+            }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (rk[k] >= 0) at(base + nk - 1 - k) = rk[k];
+        }
         sp += pushed;
         if (sp == 0) tdone = true;
       }

@@ -121,8 +121,8 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
       const int k0 = lane - gbase, m = tdone || done ? 0 : min(sp, sp > grows / 2 ? 1 : gsize);
       const bool act = k0 < m;
       if (act) {
-        const int i = sp - 1 - k0;
-        node = i < grows ? at(i) : deep[i - grows];
+        if (__builtin_expect(sp > grows, 0)) node = deep[sp - 1 - grows];
+        else node = at(sp - 1 - k0);
       }
       sp -= m;
       float tk[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
@@ -166,13 +166,19 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
         tdone = true;
         nq = 0;
       } else if (m > 0) {
+        if (__builtin_expect(sp + pushed > grows, 0)) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (rk[k] >= 0) {  // hits are sorted first
-            const int i = base + nk - 1 - k;
-            if (i < grows) at(i) = rk[k];
-            else deep[i - grows] = rk[k];
-          }
+          for (int k = 0; k < 4; ++k)
+            if (rk[k] >= 0) {  // hits are sorted first
+              const int i = base + nk - 1 - k;
+              if (i < grows) at(i) = rk[k];
+              else deep[i - grows] = rk[k];
+            }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (rk[k] >= 0) at(base + nk - 1 - k) = rk[k];
+        }
         sp += pushed;
         if (sp == 0) tdone = true;
       }
