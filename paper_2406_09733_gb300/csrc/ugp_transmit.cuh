@@ -29,11 +29,12 @@ constexpr int kTrLeafQ = 10;  // primitives a lane may hold back (top of its sta
 // With kOneScene all rays share the scene, whose fields then come from the constant bank.
 //
 // `P` collects the hits:
-//   leaf(bool ok, const PrimHit& h, int o, bool work, int off, int mine)   called by all lanes in a leaf
-//       step: this lane's primitive is hit (ok) by the ray of lane o; `work` lanes took a primitive, those
-//       of one ray are neighbours; this lane's own ray's start at lane off, `mine` of them were waiting
+//   leaf(bool ok, const PrimHit& h, int o, int off, int mine)   called by all lanes in a leaf step: this lane's
+//       primitive is hit (ok) by the ray of lane o; those of one ray are on neighbouring lanes, this lane's
+//       own ray's from lane off on, of the `mine` that were waiting as many as there are lanes
 //   bool enough()    after it, by lanes whose primitives were taken: nothing more can matter
 //   kNearFirst       children are visited nearest first
+//   kInOrder         a ray's primitives are handed to leaf() in the order in which the ray met them
 static_assert(kTrLeafQ < 16, "queue lengths are summed from four bit planes");
 //
 // With kGroup, 1 << lg neighbouring lanes share a ray (its arguments are the same on all of them): the
@@ -104,12 +105,14 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
         k2 = __shfl_sync(mask, k2, o);
       }
       PrimHit h;
-      const int slot = work ? lq[(nq_o - 1 - (lane - off_o)) * stride + (o - lane)] : 0;
+      const int slot = work ? lq[(P::kInOrder ? lane - off_o : nq_o - 1 - (lane - off_o)) * stride + (o - lane)] : 0;
       const bool ok = prim_test_of<true>(work, prims, wlo, slot, ro, t0o, t1o, k2, exo, h);
-      pol.leaf(ok, h, o, work, off, mine);
+      pol.leaf(ok, h, o, off, mine);
       __syncwarp(mask);
       if (kGroup || mine > 0) {
         nq = mine - min(mine, max(0, 32 - off));
+        if (P::kInOrder && nq > 0 && nq < mine)  // at most one ray keeps some, the last that had its turn
+          for (int k = 0; k < nq; ++k) lq[k * stride] = lq[(k + mine - nq) * stride];
         if (pol.enough()) {
           done = true;
           nq = 0;
@@ -270,12 +273,12 @@ static __device__ __forceinline__ void tr_walk(const TraceScene& sc, const Ray& 
 // `acc` points at this thread's entry of a shared array of sums; each lane of a leaf step adds its
 // primitive's term to the owner's with a shared-memory atomic. Other arguments as for tr_walk.
 struct DepthSum {
-  static constexpr bool kNearFirst = true;
+  static constexpr bool kNearFirst = true, kInOrder = false;
   static constexpr float kScale = 1099511627776.f;  // 2^40
   static constexpr unsigned long long kOne = 1ull << 40;
   unsigned long long* acc;  // the warp's sums; a group's is its first lane's
   int first;                // ~(lanes per ray - 1)
-  __device__ void leaf(bool ok, const PrimHit& h, int o, bool, int, int) {
+  __device__ void leaf(bool ok, const PrimHit& h, int o, int, int) {
     if (ok)
       atomicAdd(acc + (o & first),
                 (unsigned long long)__float2ll_rn(fminf(fmaxf(hit_half_integral(h), 0.f), 2.f) * kScale));
