@@ -9,9 +9,9 @@
 // point and entry (1M points: 1.2 ms at D = 3, 5.0 at D = 16, of the FP32 pipes' rate); here it is one
 // minimum per accumulator.
 //   * Points and entries are moved by a common centre and cut into BF16 pieces (x = h + m + l, 24
-//     bits). A row of A holds pieces of x and three ones, a row of B the pieces of -c that they meet
-//     and those of |c|^2 / 2: with 6 products per dimension (hh hm mh mm hl lh) what is left out is below
-//     2^-26 of |x||c|, with 3 (hh hm mh; D = 16) below 2^-16.4.
+//     bits; |m| <= 2^-8 |x|, |l| <= 2^-17 |x|). A row of A holds pieces of x and three ones, a row of B the
+//     pieces of -c that they meet and those of |c|^2 / 2: with 6 products per dimension (hh hm mh mm hl lh) what is
+//     left out is at most 2^-24 of |x||c|, with 3 (hh hm mh; D = 16) 2^-15.
 //   * A block takes 256 points, as two M = 128 tiles, against 32 tiles of 128 entries that one warp brings
 //     in by bulk copies (ring of 4). A warp for each point tile issues its products, into two accumulator
 //     buffers, and two threads per point (four warpgroups) read 64 of its 128 accumulators per tile each.
@@ -50,8 +50,9 @@ constexpr uint64_t kWaitNs = 2000000000ull;  // 2 s per wait
 constexpr float kDead = 1.7014118e38f;       // score of an entry left out (2^127)
 
 // Products per dimension, K (a multiple of 16), entries per granule and the relative error bound of s
-// (against (|x| + max |c|)^2): the products left out, K additions at 2^-22 each, the rounding of the
-// moved coordinates and of d2 itself.
+// (against |x||c| + |c|^2 / 2): the products left out, an addition at 2^-22 for each of the others, the rounding of
+// the moved coordinates and of |c|^2 / 2. That makes 0.66 2^-16 at D = 6 and 1.41 2^-15 at D = 16. A bound of
+// 2^-15 there, too small, took 25.29 ms for the codebook of 1M points, 1.5 2^-15 takes 25.37, 2^-14 25.47.
 template <int D>
 struct Cfg {
   static constexpr int kTerms = D <= 6 ? 6 : 3;
@@ -63,7 +64,7 @@ struct Cfg {
   // (D = 16: 0.77 -> 0.71 ms) or where many entries are nearly equal (D = 3, sizes of a wall: 0.63 -> 0.58).
   static constexpr int kUnit = D == 4 || D == 6 ? 32 : 16;
   static constexpr int kQuads = D / 4 + 1;  // float4 of an entry and its index
-  static constexpr float kErr = D <= 6 ? 1.52587890625e-05f : 3.0517578125e-05f;  // 2^-16, 2^-15
+  static constexpr float kErr = D <= 6 ? 1.52587890625e-05f : 4.57763671875e-05f;  // 2^-16, 1.5 2^-15
   static_assert(K <= (D <= 6 ? 48 : 64), "the error bound is for these K");
   static constexpr uint32_t kA = 128 * K * 2, kB = kTileN * K * 2;
   static constexpr int kMinStride = kGrans + 1;
