@@ -14,39 +14,31 @@ struct t3 {
   float a, b, c;
 };
 
-#ifdef __CUDA_ARCH__
+// not contracted into fmas
 __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-#define UGP_SPLIT_FN __device__ __forceinline__
-#else
-// the same arithmetic on the host (for checks); not contracted, as each is a call of its own
-inline float add(float a, float b) { volatile float r = a + b; return r; }
-inline float sub(float a, float b) { volatile float r = a - b; return r; }
-inline float mul(float a, float b) { volatile float r = a * b; return r; }
-#define UGP_SPLIT_FN inline
-#endif
 
-UGP_SPLIT_FN void two_sum(float a, float b, float& s, float& e) {
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = add(a, b);
   const float bb = sub(s, a);
   e = add(sub(a, sub(s, bb)), sub(b, bb));
 }
-UGP_SPLIT_FN void two_prod(float a, float b, float& p, float& e) {
+__device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
   p = mul(a, b);
   e = fmaf(a, b, -p);
 }
-UGP_SPLIT_FN t3 renorm(float a, float b, float c) {
+__device__ __forceinline__ t3 renorm(float a, float b, float c) {
   float s, t, u, v, w;
   two_sum(b, c, s, t);
   two_sum(a, s, u, v);
   two_sum(v, t, w, c);
   return {u, w, c};
 }
-UGP_SPLIT_FN t3 neg(t3 x) { return {-x.a, -x.b, -x.c}; }
+__device__ __forceinline__ t3 neg(t3 x) { return {-x.a, -x.b, -x.c}; }
 
 // p q + r s of floats.
-UGP_SPLIT_FN t3 dot2(float p, float q, float r, float s) {
+__device__ __forceinline__ t3 dot2(float p, float q, float r, float s) {
   float ph, pl, rh, rl, h, e, l, f, m, g;
   two_prod(p, q, ph, pl);
   two_prod(r, s, rh, rl);
@@ -55,21 +47,21 @@ UGP_SPLIT_FN t3 dot2(float p, float q, float r, float s) {
   two_sum(e, l, m, g);
   return renorm(h, m, add(g, f));
 }
-UGP_SPLIT_FN t3 add3(t3 x, t3 y) {
+__device__ __forceinline__ t3 add3(t3 x, t3 y) {
   float s, e, t, f, m, g;
   two_sum(x.a, y.a, s, e);
   two_sum(x.b, y.b, t, f);
   two_sum(e, t, m, g);
   return renorm(s, m, add(add(g, f), add(x.c, y.c)));
 }
-UGP_SPLIT_FN t3 mulf(t3 x, float m) {
+__device__ __forceinline__ t3 mulf(t3 x, float m) {
   float p, e, q, g, s, t;
   two_prod(x.a, m, p, e);
   two_prod(x.b, m, q, g);
   two_sum(e, q, s, t);
   return renorm(p, s, add(add(t, g), mul(x.c, m)));
 }
-UGP_SPLIT_FN t3 mul3(t3 x, t3 y) {
+__device__ __forceinline__ t3 mul3(t3 x, t3 y) {
   float p, e, q, g, h, k, s, t, u, v;
   two_prod(x.a, y.a, p, e);
   two_prod(x.a, y.b, q, g);
@@ -80,7 +72,7 @@ UGP_SPLIT_FN t3 mul3(t3 x, t3 y) {
   return renorm(p, u, add(add(add(t, v), add(g, k)), c));
 }
 // 1 / x by the series of r0 / (1 - e), e = 1 - x r0 with r0 = 1 / x.a rounded (|e| <= 2^-23).
-UGP_SPLIT_FN t3 recip3(t3 x) {
+__device__ __forceinline__ t3 recip3(t3 x) {
   const float r0 = 1.f / x.a;
   const float e0 = fmaf(-x.a, r0, 1.f);  // exact
   float q, g, E, f, p, pe;
@@ -96,8 +88,8 @@ UGP_SPLIT_FN t3 recip3(t3 x) {
 // need not have unit length, as hi + lo, and g0 = mag / ((2 pi)^(3/2) s_x s_y s_z). The quaternion and
 // the scales enter by their mantissas (powers of two are exact), so nothing over- or underflows
 // on the way.
-UGP_SPLIT_FN void whitening(float w, float x, float y, float z, const float s[3], float mag, float hi[9], float lo[9],
-                            float& g0) {
+__device__ __forceinline__ void whitening(float w, float x, float y, float z, const float s[3], float mag, float hi[9],
+                                          float lo[9], float& g0) {
   int eq, em;
   frexpf(fmaxf(fmaxf(fabsf(w), fabsf(x)), fmaxf(fabsf(y), fabsf(z))), &eq);
   const float sc = ldexpf(1.f, -eq);
