@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(256) k_collapse4(int n_int, const float4* __re
   q[3] = make_uint4(uint32_t(r4[0]), uint32_t(r4[1]), uint32_t(r4[2]), uint32_t(r4[3]));
 }
 
-__global__ void k_init_bounds(int* bounds, int* n_flags_zero_dummy) {
+__global__ void k_init_bounds(int* bounds) {
   if (threadIdx.x < 6) bounds[threadIdx.x] = f2o(3.0e38f);
 }
 
@@ -569,7 +569,7 @@ extern "C" ugp_status ugp_build_bvh(const ugp_prims* prims, float cutoff_eps, vo
   const unsigned G = unsigned((n + T - 1) / T);
   prof_begin(kStBuild, st);
   UGP_CUDA_CHECK(cudaMemsetAsync(ws + L.bounds, 0, 64, st));
-  k_init_bounds<<<1, 32, 0, st>>>(bounds, nullptr);
+  k_init_bounds<<<1, 32, 0, st>>>(bounds);
   k_prim_bounds<<<G < unsigned(kBoundsBlocks) ? G : unsigned(kBoundsBlocks), T, 0, st>>>(n, prims->mean3, prims->quat4, prims->scale3, prims->magnitude, b->k,
                                  aabb, bounds, n_invalid);
   UGP_CUDA_CHECK(cudaGetLastError());

@@ -422,7 +422,7 @@ __device__ __forceinline__ void write_out(const Outputs& O, int idx, const Finis
   }
 }
 
-// Appends slot j of the table to the list of a bigger pass (counter `count`, array `list`).
+// Appends slot j of the table to the list of the second pass (counter `count`, array `list`).
 __device__ __forceinline__ void hand_on(int* count, int* list, int j) { list[atomicAdd(count, 1)] = j; }
 
 // Bound by instruction issue (60% of the slots) and the latency of its dependent steps, so resident
@@ -480,11 +480,10 @@ __global__ void __launch_bounds__(32 * kDWarps, 6) k_dense(TraceScene sc0, Dense
 
 // The rays the first pass handed on (count of them in `list`), one warp each, kWarps warps per
 // block, up to kCap intervals per ray in the warp's slot of q.big_iv; a ray with more has its
-// bracket narrowed by sub-bins (or is handed on to a next pass when `next_count` is given).
+// bracket narrowed by sub-bins.
 template <int kCap, int kWarps>
 __global__ void __launch_bounds__(32 * kWarps, 4) k_dense_big(TraceScene sc0, DenseQueue q, const int* count_p,
-                                                           const int* __restrict__ list, int* next_count,
-                                                           int* __restrict__ next_list, Outputs O) {
+                                                           const int* __restrict__ list, Outputs O) {
   extern __shared__ __align__(16) unsigned char dsm[];
   WarpSmemBig& W = reinterpret_cast<WarpSmemBig*>(dsm)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -501,7 +500,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_dense_big(TraceScene sc0, De
     uint8_t st = UGP_RAY_OK;
     unsigned nn = 0, np = 0;
     Finish f{-1, R.t1, R.t1, UGP_RAY_OK};
-    bool done = false, handed = false;
+    bool done = false;
     for (int level = 0; level < kDLevels && !done && st == UGP_RAY_OK; ++level) {
       // ---- 1. collect the intervals meeting [lo, hi]
       int n = 0;
@@ -521,9 +520,6 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_dense_big(TraceScene sc0, De
         // ---- 2. the solve
         f = solve(gw, iv, n, lo, hi, Flo, R.u, R.u2, R.t1, O.spawn_mode, true);
         done = true;
-      } else if (next_count && level == 0) {
-        handed = true;  // the next pass holds more intervals
-        break;
       } else {
         // ---- 3. too many intervals: shrink the bracket to the crossing sub-bin
         W.bin[lane] = 0ull;
@@ -577,17 +573,6 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_dense_big(TraceScene sc0, De
       }
     }
     const unsigned tn = gw.total(nn), tp = gw.total(np);
-    if (handed) {
-      if (lane == 0) {
-        hand_on(next_count, next_list, j);
-        if (O.stats) {
-          atomicAdd(O.stats + 0, (unsigned long long)tn);
-          atomicAdd(O.stats + 1, (unsigned long long)tp);
-        }
-      }
-      __syncwarp();
-      continue;
-    }
     if (st != UGP_RAY_OK) f.st = st;
     else if (!done) f.st = UGP_RAY_ITER_LIMIT;
     if (lane == 0) {
@@ -643,7 +628,7 @@ ugp_status launch_dense(const TraceScene& sc, const DenseQueue& q, int64_t n_hos
   k_dense_big<kBigCap, kWideWarps><<<cap_grid((max_slots + kWideWarps - 1) / kWideWarps,
                                               g_wide_grid < slot_blocks ? g_wide_grid : slot_blocks),
                                      32 * kWideWarps, sizeof(WarpSmemBig) * kWideWarps, stream>>>(
-      sc, q, q.count + 2, q.wide, nullptr, nullptr, O);
+      sc, q, q.count + 2, q.wide, O);
   prof_end(kStDense, stream, 2);
   UGP_CUDA_CHECK(cudaGetLastError());
   return UGP_OK;
