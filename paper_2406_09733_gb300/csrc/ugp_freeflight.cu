@@ -82,7 +82,7 @@ ugp_status launch_free_flight(const TraceScene& sc, int64_t n, const float* o3, 
   int* next = dq.count + 1;  // the scan's ray counter, in the queue header next to the queue length
   UGP_CUDA_CHECK(cudaMemsetAsync(dq.count, 0, 4 * sizeof(int), stream));
   // the statistics count whole rays per lane
-  const auto kern = ctr ? k_free_flight<true, false> : (n <= kFFFew ? k_free_flight<false, true> : k_free_flight<false, false>);
+  const auto kern = ctr ? k_free_flight<true, false> : (ff_few(n, sc.n_prims) ? k_free_flight<false, true> : k_free_flight<false, false>);
   const int64_t need = (n + kFFBlock / 32 - 1) / (kFFBlock / 32);  // down to one ray per warp (rays_per_warp)
   const int cap = scan_grid((const void*)kern);
   const unsigned grid = unsigned(need < cap ? need : cap);

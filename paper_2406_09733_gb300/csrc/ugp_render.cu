@@ -642,11 +642,11 @@ extern "C" ugp_status ugp_render(const ugp_bvh* bvh, const ugp_materials* materi
       UGP_CUDA_CHECK(cudaMemsetAsync(gs.L.c[9], 0, size_t(RL.E) * 4, st));
   }
   const int g_cam = grid_for((const void*)k_camera, 256, n);
-  const auto extend = n <= kFFFew && !stats ? k_extend<true> : k_extend<false>;
+  const auto extend = ff_few(n, sc.n_prims) && !stats ? k_extend<true> : k_extend<false>;
   const int g_ext = grid_for((const void*)extend, kFFBlock, 32 * n);  // down to one ray per warp
   const int g_shade = guide ? grid_for((const void*)k_shade<true>, kShadeBlock, n) : grid_for((const void*)k_shade<false>, kShadeBlock, n);
   // small images: groups of lanes per ray (the statistics count whole rays per lane)
-  const bool few = n <= kTrFew && !stats;
+  const bool few = tr_few(n, sc.n_prims) && !stats;
   const int g_shadow = few ? tr_few_grid(n) : tr_grid(n);
   const auto shadow = few ? k_shadow<true> : k_shadow<false>;
   const int g_acc = grid_for((const void*)k_accumulate, 256, n);

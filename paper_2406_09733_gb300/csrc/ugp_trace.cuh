@@ -57,6 +57,11 @@ constexpr int kTrFew = 72 * kTrWarps;
 __host__ __device__ constexpr int tr_group(int64_t n) {
   return n <= kTrWarps ? 5 : (2 * n <= 5 * kTrWarps ? 4 : (n <= 16 * kTrWarps ? 3 : (n <= kTrFew ? 2 : 0)));
 }
+// Whether n rays of a scene of n_prims go in groups: in a scene of few primitives the chains are short, and a group's
+// lanes find nothing to do. Transmittances, us, in groups and a lane each: 16 primitives and 150,000 rays 41 and 19,
+// 64 and 150,000 55 and 41, 128 and 150,000 76 and 66, 300 and 300,000 234 and 200; 64 and 20,000 17 and 22 (64 and 40,000
+// 29 and 22), 128 and 40,000 28 and 40.
+inline bool tr_few(int64_t n, int64_t n_prims) { return n <= kTrFew && n <= 600 * n_prims; }
 // Blocks of a launch of up to n <= kTrFew rays in groups.
 inline int tr_few_grid(int64_t n) {
   int64_t t = n << tr_group(n);  // lanes; a smaller count may take more of them
@@ -80,6 +85,9 @@ constexpr int kFFFew = 60 * kFFWarps;
 __host__ __device__ constexpr int ff_group(int64_t n) {
   return n <= 3 * kFFWarps ? 5 : (n <= 10 * kFFWarps ? 4 : (n <= 25 * kFFWarps ? 3 : (n <= kFFFew ? 2 : 0)));
 }
+// As tr_few; free flights, us: 16 primitives and 40,000 rays 73 and 47, 64 and 150,000 189 and 116, 128 and 80,000
+// 143 and 116, 300 and 150,000 342 and 254; 64 and 10,000 50 and 81, 300 and 80,000 205 and 232.
+inline bool ff_few(int64_t n, int64_t n_prims) { return n <= kFFFew && n <= 12000 + 250 * n_prims; }
 
 // Blocks of a transmittance launch of up to n rays.
 inline int tr_grid(int64_t n) {
