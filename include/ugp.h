@@ -638,8 +638,11 @@ ugp_status ugp_render_batch_autotune(int32_t n_req, const ugp_request* reqs, int
  *   overflowed slot list)
  * for free-flight and transmittance queries (standalone, and the renderer's extend
  * pass), and the first five quantities at [6..10] for the renderer's shadow rays;
- * [11] is reserved.  NULL turns counting off (the default).  Host-side
- * setting, not thread safe against concurrent tracing calls. */
+ * [11] is reserved.  While counting, calls of few rays run with a lane per ray, as
+ * larger ones do, in place of a group of lanes (which visits a few more nodes), so their
+ * counts and times are those of that kernel; the results are the same.  NULL turns
+ * counting off (the default).  Host-side setting, not thread safe against concurrent
+ * tracing calls. */
 ugp_status ugp_set_trace_counters(unsigned long long* counters);
 
 /* ------------------------------------------------------------------ measurement
