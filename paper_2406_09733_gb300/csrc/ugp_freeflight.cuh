@@ -748,19 +748,13 @@ __device__ void scan_groups(FFSmem<kFFStack>& sm, Src& src, int* next, int lg) {
         tdone = true;
         nq = 0;
       } else if (m > 0) {
-        if (__builtin_expect(sp + pushed > grows, 0)) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (rk[k] >= 0) {  // hits are sorted first; the nearest on top
-              const int i = base + nk - 1 - k;
-              if (i < grows) at(i) = rk[k];
-              else deep[i - grows] = rk[k];
-            }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (rk[k] >= 0) at(base + nk - 1 - k) = rk[k];
-        }
+        for (int k = 0; k < 4; ++k)
+          if (rk[k] >= 0) {  // hits are sorted first; the nearest on top
+            const int i = base + nk - 1 - k;
+            if (i < grows) at(i) = rk[k];
+            else deep[i - grows] = rk[k];
+          }
         sp += pushed;
         if (sp == 0) tdone = true;
       }
