@@ -472,7 +472,7 @@ __device__ void scan_persistent(FFSmem<kStack>& sm, Src& src, int* next) {
         nq = 0;
       } else if (nk > 0) {
         // the farther children go on the stack, farthest first, so the nearer pop first
-        if (sp + nk - 1 > kStack) {  // rare
+        if (sp + nk - 1 > kStack) {  // rare, and apart: compared at each push, a 1920 x 1080 frame took 0.8% longer
           if (sp + nk - 1 > kStackMax) {
             c.st = UGP_RAY_STACK_OVERFLOW;
             tdone = true;

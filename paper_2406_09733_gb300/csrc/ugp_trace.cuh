@@ -24,7 +24,8 @@ constexpr int kTrWarps = 152 * kTrBlocksPerSM * kTrBlock / 32;  // warps of the 
 // Rays a warp takes when n of them are spread over `warps` resident warps (1 to 32). A launch with
 // fewer rays than the GPU has lanes is bound by the longest chain of steps in a warp, and a step
 // takes the longer the more rays share it, while idle lanes still take the leaf steps' primitives:
-// so the rays are spread over all resident warps, down to one each. Scan and transmittance of 2,048
+// so the scan, the renderer's shadow rays and the radiance field spread theirs over all resident warps, down to one
+// each (transmittance queries of few rays go in groups of lanes instead, below). Scan and transmittance of 2,048
 // rays through 1,000 primitives: 396 us at 32 rays per warp (most warps idle), 275 at 16 or more, 227 at
 // 8, 199 at 4, 189 at 2, 184 at 1; a 128 x 128 render of that scene, 4 spp at depth 4: 4.63 ms -> 2.37.
 __host__ __device__ constexpr int rays_per_warp(int64_t n, int64_t warps) {
