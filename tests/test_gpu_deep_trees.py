@@ -73,7 +73,7 @@ def test_small_and_large_calls_agree(env, kind, n):
 
 @pytest.mark.parametrize("kind", ["decades", "plume"])
 def test_radiance_field_reaches_every_primitive(env, kind):
-    """With emission 1 and background 1 a ray sees 1 whatever it meets."""
+    """With emission 1 and no background an unsaturated ray sees 1 - T."""
     torch, ugp, _, scene = env
     bvh, rays, _, em, full = scene(kind)
     rgb, st = ugp.render_radiance_field(bvh, *rays, torch.ones_like(em), (0.0, 0.0, 0.0))
